@@ -895,55 +895,56 @@ __global__ void k_clear_mr(Sys* sys, int B) {
 // ---- FGMRES(m) vector kernels ---------------------------------------------------------------
 // Arnoldi step j works on the basis V[0..j] (vector i of system b at V + (i*B + b)*ne) and the
 // new vector w = V[j+1].  Partial slot layout: 2*(j+1) doubles (re, im of <V_i, w>) per block.
-template <typename T>
-__device__ inline void warp_accum(T re, T im, double* slot_re, double* slot_im) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    re += __shfl_xor_sync(0xffffffffu, re, o);
-    im += __shfl_xor_sync(0xffffffffu, im, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    *slot_re += (double)re;
-    *slot_im += (double)im;
-  }
-}
-
 #define FG_MAXV 65  // m + 1 <= 65
 
-// The last block of an orthogonalisation kernel to finish (per system b; cnt counts the finished blocks
-// and is reset by the last one) sums the nq per-block partials in a fixed order:
-// one warp per coefficient q, its lanes taking blocks lane, lane + 32, ..., then a shuffle tree.
-// Returns true in the last block (all of its threads), with hout[b][0 .. nq-1] written.
-__device__ inline bool fg_last_block_fin(const double* part, int nq, double* hout, unsigned* cnt, int b, const P& p) {
-  __shared__ int last;
-  __threadfence();  // every thread's partials are visible before the block's arrival is counted
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&cnt[b], 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const double* pb = part + (long long)b * p.nblk * p.pstride;
-  for (int q = warp; q < nq; q += nw) {
-    double sum = 0.0;
-    for (int k = lane; k < p.nblk; k += 32) sum += __ldcg(pb + (long long)k * p.pstride + q);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) hout[(long long)b * 2 * FG_MAXV + q] = sum;
-  }
-  __threadfence_block();
-  __syncthreads();
-  if (threadIdx.x == 0) cnt[b] = 0u;
-  return true;
+// Partial sums of an orthogonalisation pass: value q of block k of system b at b * nblk * pstride +
+// q * gridDim.x + k, each value's partials one contiguous run.  k_fg_fin sums them, one block per value, in
+// FP64 and in a fixed order.  GB300 adds two FP64 numbers per clock and SM: the last block of a pass
+// summing all 2 nv values by itself took 35 us of a 66 us pass at 64^3 and nv = 31 (608 partials a value);
+// spread over the SMs it is a launch of 3 us.
+__device__ inline double* fg_slot(double* part, const P& p, int b, int q) {
+  return part + (long long)b * p.nblk * p.pstride + (long long)q * gridDim.x + blockIdx.x;
 }
 
-// Hessenberg column j = h + h2, h_{j+1,j} = ||w||; Givens rotations; residual estimate |g_{j+1}|
-__device__ inline void fg_givens(int b, const double* __restrict__ hn2, int j, const double* __restrict__ h1,
-                                 const double* __restrict__ h2, double* H, double* G, double* CS, double* SN, Sys* sys,
-                                 const P& p) {
+// sum of in[0 .. n-1] by a block of NT threads, every thread receives it
+template <int NT>
+__device__ inline double fg_block_sum(const double* in, int n) {
+  __shared__ double ws[NT / 32];
+  double sum = 0.0;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < n; k += NT) sum += in[k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  sum = ws[0];
+#pragma unroll
+  for (int k = 1; k < NT / 32; ++k) sum += ws[k];
+  return sum;
+}
+
+__global__ void __launch_bounds__(128) k_fg_fin(const double* __restrict__ part, int nb, double* hout,
+                                                const Sys* __restrict__ sys, P p) {
+  const int b = blockIdx.y, q = blockIdx.x;
+  if (sys[b].inner_status != SYS_RUN) return;
+  const double sum = fg_block_sum<128>(part + (long long)b * p.nblk * p.pstride + (long long)q * nb, nb);
+  if (threadIdx.x == 0) hout[(long long)b * 2 * FG_MAXV + q] = sum;
+}
+
+// The third pass's end, one block per system: ||w||^2 from its nb partials; Hessenberg column j = h + h2,
+// h_{j+1,j} = ||w||; the earlier Givens rotations and the new one; residual estimate |g_{j+1}|.
+// The rotations (c_i complex, s_i real) run down the column as lo_{i+1} = c_i h_{i+1} - s_i lo_i and give
+// H_i = conj(c_i) lo_i + s_i h_{i+1}: only s_i lo_i is a chain, all else is done for every i at once (as one
+// chain of complex products FP64 latency made it 29 us at j = 30).
+__global__ void __launch_bounds__(256) k_fg_givens(const double* __restrict__ part, int nb, int j,
+                                                   const double* __restrict__ h1, const double* __restrict__ h2,
+                                                   double* H, double* G, double* CS, double* SN, int* mirror, Sys* sys,
+                                                   P p) {
+  __shared__ double2 hi[FG_MAXV], tc[FG_MAXV], lo[FG_MAXV];
+  __shared__ double rs[FG_MAXV], quot[4];
+  const int b = blockIdx.x, i = threadIdx.x;
   Sys& s = sys[b];
   if (s.inner_status != SYS_RUN) return;
-  const double nrm2 = hn2[(long long)b * 2 * FG_MAXV];  // ||w||^2, reduced by the last block
   const int m = p.m;
   double2* Hc = (double2*)(H + (long long)b * 2 * (m + 1) * m) + (long long)j * (m + 1);  // column j
   double2* g = (double2*)(G + (long long)b * 2 * (m + 1));
@@ -951,208 +952,232 @@ __device__ inline void fg_givens(int b, const double* __restrict__ hn2, int j, c
   double2* sn = (double2*)(SN + (long long)b * 2 * m);
   const double2* a1 = (const double2*)(h1 + (long long)b * 2 * FG_MAXV);
   const double2* a2 = (const double2*)(h2 + (long long)b * 2 * FG_MAXV);
-  for (int i = 0; i <= j; ++i) Hc[i] = cadd(a1[i], a2[i]);
-  const double hn = sqrt(nrm2);
-  Hc[j + 1] = make_double2(hn, 0.0);
-  if (!isfinite(hn) || !cfinite(Hc[j])) { s.inner_status = SYS_NAN; return; }
-  for (int i = 0; i < j; ++i) {
-    double2 hi = Hc[i], hi1 = Hc[i + 1];
-    Hc[i] = cadd(cmul(cconj(cs[i]), hi), cmul(cconj(sn[i]), hi1));
-    Hc[i + 1] = csub(cmul(cs[i], hi1), cmul(sn[i], hi));
+  double2 rc = make_double2(0.0, 0.0);
+  if (i <= j) hi[i] = cadd(a1[i], a2[i]);
+  if (i < j) {
+    rc = cs[i];
+    rs[i] = sn[i].x;
   }
-  double2 a = Hc[j], c = Hc[j + 1];
-  double den = sqrt(cabs2(a) + cabs2(c));
-  if (den > 0.0) {
-    cs[j] = make_double2(a.x / den, a.y / den);
-    sn[j] = make_double2(c.x / den, c.y / den);
-  } else {
-    cs[j] = make_double2(1.0, 0.0);
-    sn[j] = make_double2(0.0, 0.0);
+  const double hn = sqrt(fg_block_sum<256>(part + (long long)b * p.nblk * p.pstride, nb));  // (has a barrier)
+  if (!isfinite(hn) || !cfinite(hi[j])) {  // uniform over the block
+    __syncthreads();
+    if (i == 0) mirror[b] = s.inner_status = SYS_NAN;
+    return;
   }
-  Hc[j] = make_double2(den, 0.0);
-  Hc[j + 1] = make_double2(0.0, 0.0);
-  double2 gj = g[j];
-  g[j + 1] = make_double2(-(sn[j].x * gj.x - sn[j].y * gj.y), -(sn[j].x * gj.y + sn[j].y * gj.x));
-  g[j] = cmul(cconj(cs[j]), gj);
-  s.jlast = j + 1;
-  s.inner_it += 1;
-  s.inv_hn = hn > 0.0 ? 1.0 / hn : 0.0;
-  double res2 = cabs2(g[j + 1]);
-  s.rin2 = res2;
-  if (res2 <= s.inner_tol2) s.inner_status = SYS_CONV;
-  else if (hn == 0.0 || den == 0.0) s.inner_status = SYS_CONV;  // exact invariant subspace
-  else if (j + 1 >= m || s.inner_it >= s.max_inner) s.inner_status = SYS_MAXIT;
+  if (i < j) tc[i] = cmul(rc, hi[i + 1]);
+  __syncthreads();
+  if (i == 0) {
+    double2 l = hi[0];
+    lo[0] = l;
+    for (int k = 0; k < j; ++k) {
+      l = make_double2(tc[k].x - rs[k] * l.x, tc[k].y - rs[k] * l.y);
+      lo[k + 1] = l;
+    }
+  }
+  __syncthreads();
+  const double2 a = lo[j];
+  const double den = sqrt(cabs2(a) + hn * hn);
+  if (i < 4) {  // the four divisions side by side
+    const double num = i == 0 ? a.x : (i == 1 ? a.y : (i == 2 ? hn : 1.0));
+    const double d = i < 3 ? den : hn;
+    quot[i] = d > 0.0 ? num / d : (i == 0 ? 1.0 : 0.0);
+  }
+  if (i < j) {
+    const double2 l = lo[i], h = hi[i + 1];
+    Hc[i] = make_double2(rc.x * l.x + rc.y * l.y + rs[i] * h.x, rc.x * l.y - rc.y * l.x + rs[i] * h.y);
+  }
+  if (i == j) {
+    Hc[j] = make_double2(den, 0.0);
+    Hc[j + 1] = make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  if (i == 0) {
+    const double2 cj = make_double2(quot[0], quot[1]), gj = g[j];
+    const double sj = quot[2];
+    cs[j] = cj;
+    sn[j] = make_double2(sj, 0.0);
+    const double2 gn = make_double2(-(sj * gj.x), -(sj * gj.y));
+    g[j + 1] = gn;
+    g[j] = cmul(cconj(cj), gj);
+    s.jlast = j + 1;
+    s.inner_it += 1;
+    s.inv_hn = quot[3];
+    const double res2 = cabs2(gn);
+    s.rin2 = res2;
+    if (res2 <= s.inner_tol2) s.inner_status = SYS_CONV;
+    else if (hn == 0.0 || den == 0.0) s.inner_status = SYS_CONV;  // exact invariant subspace
+    else if (j + 1 >= m || s.inner_it >= s.max_inner) s.inner_status = SYS_MAXIT;
+    mirror[b] = s.inner_status;  // the status word the next apply's predicate reads
+  }
 }
 
-// Arnoldi coefficient vectors of the orthogonalisation passes and the Hessenberg workspace, for the
-// last block's reduction and Givens step
-struct FgOut {
-  double *h1, *h2, *hn2, *H, *G, *CS, *SN;
-  unsigned* cnt;
-};
+// The three CGS2 passes over V[0..j] and the new vector w = V[j+1]:
+//   mode 0:  h_i = <V_i, w>                                (2(j+1) sums)
+//   mode 1:  w -= sum_i h_i V_i, then h2_i = <V_i, w>      (2(j+1) sums)
+//   mode 2:  w -= sum_i h2_i V_i, then ||w||^2
+//
+// complex64: one element of every vector per thread.  A tall-skinny product has as many sums as vectors
+// and millions of terms in each, so each thread keeps all of its 2 NV partial sums in registers over its
+// whole share of the elements, and nothing is exchanged between threads until the end.  The passes are
+// HBM-bound then (a few FMAs per 8 bytes), with NV independent coalesced loads in flight per thread; mode
+// 1 keeps the NV values of its element for the dot products (NV <= 32), so V is read once.  Sums run in
+// FP32 over a thread's elements and a warp's shuffles and in FP64 from there on.  NV is nv rounded up to
+// a multiple of 4; blocks of 128 threads, as many per SM as the registers of the mode allow.
+template <int NV, int MODE>
+__host__ __device__ constexpr int fg_blocks_per_sm() {
+  return NV <= 8 ? 8 : (NV <= 16 ? (MODE == 1 ? 4 : 5) : (NV <= 32 ? (NV <= 24 ? (MODE == 1 ? 3 : 4) : (MODE == 1 ? 2 : 3)) : 2));
+}
 
-// The three CGS2 passes.  They work on chunks of CH elements (one per thread, CH = 256 for complex64
-// and 128 for complex128) and keep only a few values per thread in registers:
-//   k_fg_dots:         h_i = <V_i, w>                   (2(j+1) partials per block)
-//   k_fg_update_dots:  w -= sum_i h_i V_i, then h2_i = <V_i, w>
-//   k_fg_update_norm:  w -= sum_i h2_i V_i, then ||w||^2 (partial slot 0)
-// The dots are a tall-skinny product: the chunk of w sits in shared memory and each warp streams
-// whole basis vectors (i = warp, warp + nwarps, ...) over it, summing in the vector precision within
-// the chunk and in FP64 across chunks, in a fixed order.  k_fg_update_dots keeps the chunk of every
-// V_i it reads for the update in shared memory, so V is read from HBM once for both halves.
-template <typename T>
-struct FgChunk {
-  static constexpr int CH = sizeof(T) == 4 ? 256 : 128;
-};
-
-template <typename T>
-__device__ inline void fg_chunk_dots(const typename cplx<T>::t* vchunk, long long vstride, bool vglobal,
-                                     const typename cplx<T>::t* ws, int nv, int nvalid, double* acc) {
-  constexpr int CH = FgChunk<T>::CH;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = CH / 32;
-  for (int i = warp; i < nv; i += nw) {
-    const auto* vi = vchunk + (vglobal ? (long long)i * vstride : (long long)i * CH);
-    T sr = T(0), si = T(0);
+// Sums v[0 .. 7] over the warp's 32 lanes: halving exchanges (16, 8, 4) leave every lane with one of the
+// eight values, then two more steps; lane l with l % 4 == 0 holds the sum of value (l >> 2) in the bit
+// order returned by `which`.  9 shuffles for 8 values.
+__device__ inline float warp_sum8(float (&v)[8], int lane, int* which) {
 #pragma unroll
-    for (int q0 = 0; q0 < CH; q0 += 32) {
-      const int q = q0 + lane;
-      if (q < nvalid) {
-        const auto a = vi[q], b = ws[q];
-        sr += a.x * b.x + a.y * b.y;
-        si += a.x * b.y - a.y * b.x;
+  for (int step = 0; step < 3; ++step) {
+    const int o = 16 >> step, half = 4 >> step;
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < half; ++k) {
+      const float send = up ? v[k] : v[k + half];
+      const float keep = up ? v[k + half] : v[k];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  float t = v[0];
+  t += __shfl_xor_sync(0xffffffffu, t, 2);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  *which = ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0);
+  return t;
+}
+
+template <int NV, int MODE>
+__global__ void __launch_bounds__(128, (fg_blocks_per_sm<NV, MODE>())) k_fg_stream(
+    const float2* __restrict__ Vb, float2* __restrict__ w, int nv, const double* __restrict__ hcoef,
+    const Sys* __restrict__ sys, double* part, P p) {
+  static_assert(NV % 4 == 0 && NV <= 64 && (MODE == 0 || MODE == 1), "sums come in groups of eight");
+  constexpr bool KEEP = MODE == 1 && NV <= 32;  // the element of every vector stays in registers
+  const int b = blockIdx.y;
+  if (sys[b].inner_status != SYS_RUN) return;
+  __shared__ float2 hs[NV];
+  __shared__ float red[4][2 * NV];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
+  const float2* v0 = Vb + off;
+  w += off;
+  if (MODE == 1) {
+    for (int i = tid; i < NV; i += 128)
+      hs[i] = i < nv ? make_float2((float)hcoef[(long long)b * 2 * FG_MAXV + 2 * i],
+                                   (float)hcoef[(long long)b * 2 * FG_MAXV + 2 * i + 1])
+                     : make_float2(0.f, 0.f);
+    __syncthreads();
+  }
+  float ar[NV], ai[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) ar[i] = ai[i] = 0.f;
+  for (long long e = blockIdx.x * 128LL + tid; e < p.ne; e += (long long)gridDim.x * 128) {
+    // (the vectors' addresses by repeated addition: as i * vs the compiler keeps 2 NV registers of offsets)
+    const float2* ve = v0 + e;
+    float2 wv = w[e];
+    float2 a[KEEP ? NV : 1];
+    if (KEEP) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        a[KEEP ? i : 0] = i < nv ? *ve : make_float2(0.f, 0.f);
+        ve += vs;
       }
     }
+    if (MODE == 1) {
+      if (KEEP) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sr += __shfl_xor_sync(0xffffffffu, sr, o);
-      si += __shfl_xor_sync(0xffffffffu, si, o);
-    }
-    if (lane == 0) {
-      acc[2 * i] += (double)sr;
-      acc[2 * i + 1] += (double)si;
-    }
-  }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_fg_dots(const typename cplx<T>::t* __restrict__ Vb, int j,
-                                                 const Sys* __restrict__ sys, double* part, FgOut fo, P p) {
-  using V = typename cplx<T>::t;
-  constexpr int CH = FgChunk<T>::CH;
-  const int b = blockIdx.y;
-  if (sys[b].inner_status != SYS_RUN) return;
-  __shared__ V ws[CH];
-  __shared__ double acc[2 * FG_MAXV];
-  const int nv = j + 1, tid = threadIdx.x;
-  const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
-  const V* w = Vb + (long long)(j + 1) * vs + off;
-  for (int q = tid; q < 2 * nv; q += CH) acc[q] = 0.0;
-  for (long long c0 = (long long)blockIdx.x * CH; c0 < p.ne; c0 += (long long)gridDim.x * CH) {
-    const int nvalid = (int)min((long long)CH, p.ne - c0);
-    __syncthreads();  // the previous chunk's dots are done with ws
-    ws[tid] = tid < nvalid ? w[c0 + tid] : czero<V>();
-    __syncthreads();
-    fg_chunk_dots<T>(Vb + off + c0, vs, true, ws, nv, nvalid, acc);
-  }
-  __syncthreads();
-  double* out = part + PSLOT(p, b);
-  for (int q = tid; q < 2 * nv; q += CH) out[q] = acc[q];
-  fg_last_block_fin(part, 2 * nv, fo.h1, fo.cnt, b, p);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_fg_update_dots(const typename cplx<T>::t* __restrict__ Vb, int j,
-                                                        const double* __restrict__ hcoef,
-                                                        const Sys* __restrict__ sys, double* part, FgOut fo, P p) {
-  using V = typename cplx<T>::t;
-  constexpr int CH = FgChunk<T>::CH;
-  const int b = blockIdx.y;
-  if (sys[b].inner_status != SYS_RUN) return;
-  extern __shared__ __align__(16) unsigned char fg_smem[];
-  V* vsm = (V*)fg_smem;                 // [nv][CH]
-  const int nv = j + 1, tid = threadIdx.x;
-  V* ws = vsm + (long long)nv * CH;     // [CH]
-  double* acc = (double*)(ws + CH);     // [2 nv]
-  T* hs = (T*)(acc + 2 * nv);           // [2 nv]
-  const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
-  V* w = (V*)(Vb + (long long)(j + 1) * vs + off);
-  const double* hc = hcoef + (long long)b * 2 * FG_MAXV;
-  for (int q = tid; q < 2 * nv; q += CH) {
-    acc[q] = 0.0;
-    hs[q] = (T)hc[q];
-  }
-  for (long long c0 = (long long)blockIdx.x * CH; c0 < p.ne; c0 += (long long)gridDim.x * CH) {
-    const int nvalid = (int)min((long long)CH, p.ne - c0);
-    const bool valid = tid < nvalid;
-    __syncthreads();  // hs is set; the previous chunk's dots are done with vsm and ws
-    V wv = valid ? w[c0 + tid] : czero<V>();
-    const V* vcol = Vb + off + c0 + tid;
+        for (int i = 0; i < NV; ++i) {
+          const float2 h = hs[i], c = a[KEEP ? i : 0];
+          wv.x -= h.x * c.x - h.y * c.y;
+          wv.y -= h.x * c.y + h.y * c.x;
+        }
+      } else {
+        const float2* vi = ve;
 #pragma unroll 8
-    for (int i = 0; i < nv; ++i) {
-      const V a = valid ? vcol[(long long)i * vs] : czero<V>();
-      vsm[i * CH + tid] = a;
-      const T hr = hs[2 * i], hi = hs[2 * i + 1];
-      wv.x -= hr * a.x - hi * a.y;
-      wv.y -= hr * a.y + hi * a.x;
+        for (int i = 0; i < nv; ++i) {
+          const float2 h = hs[i], c = *vi;
+          wv.x -= h.x * c.x - h.y * c.y;
+          wv.y -= h.x * c.y + h.y * c.x;
+          vi += vs;
+        }
+      }
+      w[e] = wv;
     }
-    if (valid) w[c0 + tid] = wv;
-    ws[tid] = wv;
-    __syncthreads();
-    fg_chunk_dots<T>(vsm, 0, false, ws, nv, nvalid, acc);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      float2 c;
+      if (KEEP) {
+        c = a[KEEP ? i : 0];
+      } else {
+        c = i < nv ? *ve : make_float2(0.f, 0.f);
+        ve += vs;
+      }
+      ar[i] += c.x * wv.x + c.y * wv.y;  // conj(V_i) w
+      ai[i] += c.x * wv.y - c.y * wv.x;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NV; i += 4) {
+    float v[8] = {ar[i], ai[i], ar[i + 1], ai[i + 1], ar[i + 2], ai[i + 2], ar[i + 3], ai[i + 3]};
+    int which;
+    const float t = warp_sum8(v, lane, &which);
+    if ((lane & 3) == 0) red[warp][2 * i + which] = t;
   }
   __syncthreads();
-  double* out = part + PSLOT(p, b);
-  for (int q = tid; q < 2 * nv; q += CH) out[q] = acc[q];
-  fg_last_block_fin(part, 2 * nv, fo.h2, fo.cnt, b, p);
+  for (int q = tid; q < 2 * nv; q += 128)
+    *fg_slot(part, p, b, q) = ((double)red[0][q] + (double)red[1][q]) + ((double)red[2][q] + (double)red[3][q]);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_fg_update_norm(const typename cplx<T>::t* __restrict__ Vb, int j,
-                                                        const double* __restrict__ hcoef,
-                                                        Sys* sys, double* part, FgOut fo, P p) {
-  using V = typename cplx<T>::t;
-  constexpr int CH = FgChunk<T>::CH;
+// mode 2, complex64: the update streams the vectors eight at a time (no sums to keep)
+__global__ void __launch_bounds__(256, 5) k_fg_stream_norm(const float2* __restrict__ Vb, float2* __restrict__ w, int nv,
+                                                           const double* __restrict__ hcoef,
+                                                           const Sys* __restrict__ sys, double* part, P p) {
   const int b = blockIdx.y;
   if (sys[b].inner_status != SYS_RUN) return;
-  __shared__ T hs[2 * FG_MAXV];
-  const int nv = j + 1, tid = threadIdx.x;
+  __shared__ float2 hs[64 + 8];
+  const int tid = threadIdx.x;
   const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
-  V* w = (V*)(Vb + (long long)(j + 1) * vs + off);
-  const double* hc = hcoef + (long long)b * 2 * FG_MAXV;
-  for (int q = tid; q < 2 * nv; q += CH) hs[q] = (T)hc[q];
+  for (int i = tid; i < 64 + 8; i += 256)
+    hs[i] = i < nv ? make_float2((float)hcoef[(long long)b * 2 * FG_MAXV + 2 * i],
+                                 (float)hcoef[(long long)b * 2 * FG_MAXV + 2 * i + 1])
+                   : make_float2(0.f, 0.f);
   __syncthreads();
-  T nrm[1] = {T(0)};
-  for (long long e = (long long)blockIdx.x * CH + tid; e < p.ne; e += (long long)gridDim.x * CH) {
-    V wv = w[e];
-    const V* vcol = Vb + off + e;
-#pragma unroll 8
-    for (int i = 0; i < nv; ++i) {
-      const V a = vcol[(long long)i * vs];
-      const T hr = hs[2 * i], hi = hs[2 * i + 1];
-      wv.x -= hr * a.x - hi * a.y;
-      wv.y -= hr * a.y + hi * a.x;
+  w += off;
+  float nrm[1] = {0.f};
+  for (long long e = blockIdx.x * 256LL + tid; e < p.ne; e += (long long)gridDim.x * 256) {
+    const float2* ve = Vb + off + e;
+    float2 wv = w[e];
+    for (int i0 = 0; i0 < nv; i0 += 8) {  // (eight loads at once in the last group too)
+      float2 c[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        c[i] = i0 + i < nv ? *ve : make_float2(0.f, 0.f);
+        ve += vs;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float2 h = hs[i0 + i];
+        wv.x -= h.x * c[i].x - h.y * c[i].y;
+        wv.y -= h.x * c[i].y + h.y * c[i].x;
+      }
     }
     w[e] = wv;
     nrm[0] += wv.x * wv.x + wv.y * wv.y;
   }
-  fit_block_sum<T, 1>(nrm, part + PSLOT(p, b));
-  // the last block reduces ||w||^2 and takes the Givens step of this system
-  if (fg_last_block_fin(part, 1, fo.hn2, fo.cnt, b, p) && threadIdx.x == 0) {
-    __threadfence_block();
-    fg_givens(b, fo.hn2, j, fo.h1, fo.h2, fo.H, fo.G, fo.CS, fo.SN, sys, p);
-  }
+  fit_block_sum<float, 1>(nrm, fg_slot(part, p, b, 0));
 }
 
-
-// ---- the three CGS2 passes with bulk copies -----------------------------------------------------
-// The same passes and per-block partial layout as k_fg_dots / k_fg_update_dots / k_fg_update_norm, but
-// the block's chunk of every basis vector and of w arrives in shared memory by a bulk copy engine
-// transfer (cp.async.bulk, one 2 KB copy per vector and chunk), S chunks in flight, completed on one
-// mbarrier per stage.  The copy engine keeps the loads streaming while the threads update w and take
+// ---- complex128: the three CGS2 passes with bulk copies ------------------------------------------
+// The same passes; the block's chunk of every basis vector and of w arrives in shared memory by a bulk copy
+// engine transfer (cp.async.bulk, one 2 KB copy per vector and chunk), S chunks in flight, completed on one
+// mbarrier per stage.  (Bound by the FP64 pipe: 8 FP64 multiply-adds per 16 bytes.)  The copy engine keeps the loads streaming while the threads update w and take
 // the dot products from shared memory, so V is read from HBM once per pass at close to copy speed.
 // Dot products: warp q of NW owns the basis vectors i = q, q + NW, ...; each lane accumulates its share over
 // all of the block's chunks in the vector precision, and the warp's shuffle sum goes to the block's
-// partial slot in FP64.  Needs 16-byte aligned chunks: complex128, or complex64 with an even n_e.
+// partial slot in FP64.  Every chunk is 16-byte aligned.
 // Every wait on a stage is bounded (2^22 polls, the grid's abort word read every 4096): on a timeout the
 // block records it in the grid's error word, lets its own copies land and leaves.
 __device__ inline uint32_t kr_smem(const void* q) { return (uint32_t)__cvta_generic_to_shared(q); }
@@ -1174,12 +1199,15 @@ __device__ inline bool kr_wait(uint64_t* bar, uint32_t parity, const volatile in
   return false;
 }
 
-template <typename T, int MODE, int S>
-__global__ void __launch_bounds__(256) k_fg_cgs_bulk(const typename cplx<T>::t* __restrict__ Vb, int j,
-                                                     const double* __restrict__ hcoef, Sys* sys, double* part,
-                                                     FgOut fo, P p) {
-  using V = typename cplx<T>::t;
-  constexpr int CH = FgChunk<T>::CH;
+constexpr int FG_CH = 128;  // elements per chunk, one per thread
+
+template <int MODE, int S>
+__global__ void __launch_bounds__(FG_CH) k_fg_cgs_bulk(const double2* __restrict__ Vb, int j,
+                                                     const double* __restrict__ hcoef, const Sys* __restrict__ sys,
+                                                     double* part, P p) {
+  using T = double;
+  using V = double2;
+  constexpr int CH = FG_CH;
   constexpr int NW = CH / 32;       // warps per block (one thread per chunk element)
   constexpr int SLOTS = 64 / NW;    // basis vectors per warp: nv <= 64
   const int b = blockIdx.y;
@@ -1278,14 +1306,9 @@ __global__ void __launch_bounds__(256) k_fg_cgs_bulk(const typename cplx<T>::t* 
     __syncthreads();
     return;
   }
-  double* out = part + PSLOT(p, b);
   if (MODE == 2) {
     T v1[1] = {nrm};
-    fit_block_sum<T, 1>(v1, out);
-    if (fg_last_block_fin(part, 1, fo.hn2, fo.cnt, b, p) && tid == 0) {
-      __threadfence_block();
-      fg_givens(b, fo.hn2, j, fo.h1, fo.h2, fo.H, fo.G, fo.CS, fo.SN, sys, p);
-    }
+    fit_block_sum<T, 1>(v1, fg_slot(part, p, b, 0));
     return;
   }
 #pragma unroll
@@ -1303,69 +1326,94 @@ __global__ void __launch_bounds__(256) k_fg_cgs_bulk(const typename cplx<T>::t* 
     }
   }
   __syncthreads();
-  for (int q = tid; q < 2 * nv; q += blockDim.x) out[q] = red[q];
-  fg_last_block_fin(part, 2 * nv, MODE == 0 ? fo.h1 : fo.h2, fo.cnt, b, p);
+  for (int q = tid; q < 2 * nv; q += blockDim.x) *fg_slot(part, p, b, q) = red[q];
 }
 
-// v_{j+1} = w / h_{j+1,j}
+// v_{j+1} = w / h_{j+1,j}; with zn also the next step's preconditioned vector z_{j+1} = D^-1 v_{j+1}, while
+// v is in registers (a pass of its own read v and wrote z: 24 B per unknown, now 16)
 template <typename T>
-__global__ void __launch_bounds__(256) k_fg_scale(typename cplx<T>::t* Vb, int j, const Sys* __restrict__ sys, P p) {
+__global__ void __launch_bounds__(256) k_fg_scale(typename cplx<T>::t* Vb, int j, typename cplx<T>::t* zn,
+                                                  const typename cplx<T>::t* __restrict__ dinv,
+                                                  const Sys* __restrict__ sys, P p) {
   const int b = blockIdx.y;
   if (sys[b].inner_status != SYS_RUN) return;
-  const long long vs = (long long)p.B * p.ne;
-  auto* w = Vb + (long long)(j + 1) * vs + (long long)b * p.ne;
+  const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
+  auto* w = Vb + (long long)(j + 1) * vs + off;
   const T sc = (T)sys[b].inv_hn;
   VEC_LOOP(p) {
     auto v = w[e];
     v.x *= sc;
     v.y *= sc;
     w[e] = v;
+    if (zn) zn[off + e] = cmulv(dinv[off + e], v);
   }
 }
 
-// back substitution H y = g on the rotated (upper triangular) Hessenberg, then d = sum y_i Z_i
-__global__ void k_fg_solve(const double* __restrict__ H, const double* __restrict__ G, double* Y, const Sys* sys, P p) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= p.B) return;
+// back substitution H y = g on the rotated (upper triangular) Hessenberg, then d = sum y_i Z_i.  One warp
+// per system, two rows per lane: once y_i is known every lane takes its rows' share off at once (one thread
+// walking the triangle waited on every entry of H in turn: 155 us per cycle at m = 30).
+__global__ void __launch_bounds__(32) k_fg_solve(const double* __restrict__ H, const double* __restrict__ G, double* Y,
+                                                 const Sys* sys, P p) {
+  const int b = blockIdx.x, lane = threadIdx.x;
   const Sys& s = sys[b];
   if (s.outer_status != SYS_RUN) return;
   const int m = p.m, n = s.jlast;
   const double2* Hb = (const double2*)(H + (long long)b * 2 * (m + 1) * m);
   const double2* g = (const double2*)(G + (long long)b * 2 * (m + 1));
   double2* y = (double2*)(Y + (long long)b * 2 * FG_MAXV);
-  for (int i = n - 1; i >= 0; --i) {
-    double2 acc = g[i];
-    for (int k = i + 1; k < n; ++k) acc = csub(acc, cmul(Hb[(long long)k * (m + 1) + i], y[k]));
-    double2 hii = Hb[(long long)i * (m + 1) + i];
-    y[i] = cabs2(hii) > 0.0 ? cdiv(acc, hii) : make_double2(0.0, 0.0);
+  const double2 zero = make_double2(0.0, 0.0);
+  // rows lane and lane + 32: what is left of g, and 1 / h_ii
+  double2 acc[2], inv[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int i = lane + 32 * q;
+    acc[q] = i < n ? g[i] : zero;
+    const double2 hii = i < n ? Hb[(long long)i * (m + 1) + i] : zero;
+    inv[q] = cabs2(hii) > 0.0 ? cdiv(make_double2(1.0, 0.0), hii) : zero;
   }
-  for (int i = n; i < m; ++i) y[i] = make_double2(0.0, 0.0);
+  for (int i = n - 1; i >= 0; --i) {
+    const double2* col = Hb + (long long)i * (m + 1);
+    const double2 h0 = lane < i ? col[lane] : zero, h1 = lane + 32 < i ? col[lane + 32] : zero;
+    const double2 mine = (i >> 5) ? cmul(acc[1], inv[1]) : cmul(acc[0], inv[0]);
+    double2 yi;
+    yi.x = __shfl_sync(0xffffffffu, mine.x, i & 31);
+    yi.y = __shfl_sync(0xffffffffu, mine.y, i & 31);
+    if (lane == 0) y[i] = yi;
+    acc[0] = csub(acc[0], cmul(h0, yi));
+    acc[1] = csub(acc[1], cmul(h1, yi));
+  }
+  for (int i = n + lane; i < m; i += 32) y[i] = zero;
 }
 
-template <typename T, int MAXV>
+// d = sum_i y_i Z_i: streams the vectors eight at a time
+template <typename T>
 __global__ void __launch_bounds__(256) k_fg_combine(const typename cplx<T>::t* __restrict__ Zb, typename cplx<T>::t* d,
                                                     const double* __restrict__ Y, const Sys* __restrict__ sys, P p) {
   using V = typename cplx<T>::t;
   const int b = blockIdx.y;
   if (sys[b].outer_status != SYS_RUN) return;
+  __shared__ V ys[64 + 8];
   const int n = sys[b].jlast;
   const long long vs = (long long)p.B * p.ne;
   const long long off = (long long)b * p.ne;
   const double* y = Y + (long long)b * 2 * FG_MAXV;
-  T yr[MAXV], yi[MAXV];
-#pragma unroll
-  for (int i = 0; i < MAXV; ++i) {
-    yr[i] = i < n ? (T)y[2 * i] : T(0);
-    yi[i] = i < n ? (T)y[2 * i + 1] : T(0);
-  }
+  for (int i = threadIdx.x; i < 64 + 8; i += 256) ys[i] = i < n ? mkc<T>(y[2 * i], y[2 * i + 1]) : czero<V>();
+  __syncthreads();
   VEC_LOOP(p) {
+    const V* ze = Zb + off + e;
     V acc = czero<V>();
+    for (int i0 = 0; i0 < n; i0 += 8) {
+      V z[8];
 #pragma unroll
-    for (int i = 0; i < MAXV; ++i) {
-      if (i < n) {
-        V zi = Zb[(long long)i * vs + off + e];
-        acc.x += yr[i] * zi.x - yi[i] * zi.y;
-        acc.y += yr[i] * zi.y + yi[i] * zi.x;
+      for (int i = 0; i < 8; ++i) {
+        z[i] = i0 + i < n ? *ze : czero<V>();
+        ze += vs;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const V yi = ys[i0 + i];
+        acc.x += yi.x * z[i].x - yi.y * z[i].y;
+        acc.y += yi.x * z[i].y + yi.y * z[i].x;
       }
     }
     d[off + e] = acc;
@@ -1445,6 +1493,7 @@ namespace {
 struct Work {
   fit_grid* g = nullptr;
   int B = 0, m = 30, method = FIT_BICGSTAB, mixed = 1, pc = FIT_PC_NONE;
+  int nsm = 1;            // SMs of the device (grids of the streaming passes)
   fit_prec inner = FIT_C64;
   size_t esz = 8;         // bytes per complex inner element
   P p{};
@@ -1461,7 +1510,7 @@ struct Work {
   void* x16 = nullptr;   // U-Net input scratch ([ncell][16] bf16)
   double *part_apply = nullptr, *part_vec = nullptr;
   long long napply = 0;
-  double *h1 = nullptr, *h2 = nullptr, *hn2 = nullptr, *H = nullptr, *G = nullptr, *CS = nullptr, *SN = nullptr, *Y = nullptr;
+  double *h1 = nullptr, *h2 = nullptr, *H = nullptr, *G = nullptr, *CS = nullptr, *SN = nullptr, *Y = nullptr;
   Sys* sys = nullptr;
   Ctl* ctl = nullptr;
   unsigned* cnt = nullptr;  // per system: blocks of a vector kernel finished (last-block reductions)
@@ -1550,6 +1599,7 @@ fit_status setup(Work& w, int B) {
     ALLOC(w.x16, (size_t)g->ncell * 16 * 2);
     if ((st = fit_unet_prepare(g->unet, g, 0)) != FIT_OK) return st;
   }
+  FIT_CHECK_CUDA(cudaDeviceGetAttribute(&w.nsm, cudaDevAttrMultiProcessorCount, g->device));
   w.napply = std::max(fit_apply_partials(g, FIT_C64), fit_apply_partials(g, FIT_C128));
   ALLOC(w.part_apply, (size_t)B * w.napply * 4 * sizeof(double));
   int nblk = std::max(8, std::min(1216, (int)((ne + 255) / 256)));
@@ -1560,7 +1610,6 @@ fit_status setup(Work& w, int B) {
   if (w.method == FIT_FGMRES) {
     ALLOC(w.h1, (size_t)B * 2 * FG_MAXV * sizeof(double));
     ALLOC(w.h2, (size_t)B * 2 * FG_MAXV * sizeof(double));
-    ALLOC(w.hn2, (size_t)B * 2 * FG_MAXV * sizeof(double));
     ALLOC(w.H, (size_t)B * 2 * (w.m + 1) * w.m * sizeof(double));
     ALLOC(w.G, (size_t)B * 2 * (w.m + 1) * sizeof(double));
     ALLOC(w.CS, (size_t)B * 2 * w.m * sizeof(double));
@@ -1607,6 +1656,8 @@ struct Seq {
   double2* x;
   cudaStream_t s;
   fit_status st = FIT_OK;
+  int* mirror_inner = nullptr;  // per-system status words for the apply's predicate
+  int* mirror_outer = nullptr;
 
   dim3 vgrid() const { return dim3(w.p.nblk, w.p.B); }
   void check() {
@@ -1747,43 +1798,72 @@ struct Seq {
     fin<3>(w.part_vec, w.p.nblk, w.p.pstride, OpRho{});
   }
 
-  // the three CGS2 passes over V[0..j] (mode 0: dots; 1: update with h, dots; 2: update with h2, norm)
-  FgOut fg_out() const { return FgOut{w.h1, w.h2, w.hn2, w.H, w.G, w.CS, w.SN, w.cnt}; }
-  template <typename T, int MODE, int S>
-  void ortho_bulk(int j, const double* h) {
-    using V = typename cplx<T>::t;
-    constexpr int CH = FgChunk<T>::CH;
-    const size_t smem = (size_t)S * (j + 2) * CH * sizeof(V) + S * 8 + 2 * FG_MAXV * sizeof(T) +
-                        2 * FG_MAXV * sizeof(double);
-    auto kern = k_fg_cgs_bulk<T, MODE, S>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<vgrid(), CH, smem, s>>>((const V*)w.Vb, j, h, w.sys, w.part_vec, fg_out(), w.p);
+  // the three CGS2 passes over V[0..j] (mode 0: dots; 1: update with h, dots; 2: update with h2, norm), each
+  // followed by the sum of its nb partials per value
+  template <int MODE>
+  void ortho_fin(int j, int nb) {
+    const int nq = 2 * (j + 1);
+    if (MODE == 2)
+      k_fg_givens<<<w.p.B, 256, 0, s>>>(w.part_vec, nb, j, w.h1, w.h2, w.H, w.G, w.CS, w.SN, mirror_inner, w.sys, w.p);
+    else
+      k_fg_fin<<<dim3(nq, w.p.B), 128, 0, s>>>(w.part_vec, nb, MODE == 0 ? w.h1 : w.h2, w.sys, w.p);
     check();
   }
-  // the bulk-copy passes need 16-byte aligned chunks of every vector
-  bool bulk_ok() const { return w.esz == 16 || (w.p.ne % 2) == 0; }
+  template <int MODE, int S>
+  void ortho_bulk(int j, const double* h) {
+    const size_t smem = (size_t)S * (j + 2) * FG_CH * sizeof(double2) + S * 8 + 4 * FG_MAXV * sizeof(double);
+    auto kern = k_fg_cgs_bulk<MODE, S>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<vgrid(), FG_CH, smem, s>>>((const double2*)w.Vb, j, h, w.sys, w.part_vec, w.p);
+    check();
+    ortho_fin<MODE>(j, w.p.nblk);
+  }
+  // blocks per system of a streaming pass: the resident blocks shared by the batch, no more than the elements
+  // fill and no more than the partial-sum buffer holds
+  int stream_blocks(int per_sm, int threads) const {
+    const long long fill = (w.p.ne + threads - 1) / threads;
+    const long long res = std::max(1LL, (long long)per_sm * w.nsm / w.p.B);
+    return (int)std::max(1LL, std::min({fill, res, (long long)w.p.nblk}));
+  }
+  template <int NV, int MODE>
+  void ortho_stream(int nv, const double* h) {
+    const dim3 grid(stream_blocks(fg_blocks_per_sm<NV, MODE>(), 128), w.p.B);
+    float2* wv = (float2*)w.Vb + (size_t)nv * w.p.B * w.p.ne;
+    k_fg_stream<NV, MODE><<<grid, 128, 0, s>>>((const float2*)w.Vb, wv, nv, h, w.sys, w.part_vec, w.p);
+    check();
+    ortho_fin<MODE>(nv - 1, (int)grid.x);
+  }
   template <typename T, int MODE>
   void ortho(int j, const double* h) {
-    using V = typename cplx<T>::t;
-    constexpr int CH = FgChunk<T>::CH;
     const int nv = j + 1;
-    if (bulk_ok()) {  // three stages while they fit two blocks per SM, else two
-      if ((size_t)3 * (j + 2) * CH * sizeof(V) <= 100 * 1024) ortho_bulk<T, MODE, 3>(j, h);
-      else ortho_bulk<T, MODE, 2>(j, h);
-      return;
-    }
-    if (MODE == 0) {
-      k_fg_dots<T><<<vgrid(), CH, 0, s>>>((const V*)w.Vb, j, w.sys, w.part_vec, fg_out(), w.p);
-    } else if (MODE == 1) {
-      const size_t smem = (size_t)(nv + 1) * CH * sizeof(V) + (size_t)2 * nv * sizeof(double) +
-                          (size_t)2 * nv * sizeof(T);
-      auto kern = k_fg_update_dots<T>;
-      if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      kern<<<vgrid(), CH, smem, s>>>((const V*)w.Vb, j, h, w.sys, w.part_vec, fg_out(), w.p);
+    if constexpr (sizeof(T) == 8) {  // three stages while they fit two blocks per SM, else two
+      if ((size_t)3 * (j + 2) * FG_CH * sizeof(double2) <= 100 * 1024) ortho_bulk<MODE, 3>(j, h);
+      else ortho_bulk<MODE, 2>(j, h);
+    } else if constexpr (MODE == 2) {
+      const dim3 grid(stream_blocks(5, 256), w.p.B);
+      k_fg_stream_norm<<<grid, 256, 0, s>>>((const float2*)w.Vb, (float2*)w.Vb + (size_t)nv * w.p.B * w.p.ne, nv, h,
+                                            w.sys, w.part_vec, w.p);
+      check();
+      ortho_fin<2>(j, (int)grid.x);
     } else {
-      k_fg_update_norm<T><<<vgrid(), CH, 0, s>>>((const V*)w.Vb, j, h, w.sys, w.part_vec, fg_out(), w.p);
+      switch ((nv + 3) / 4) {
+        case 1: return ortho_stream<4, MODE>(nv, h);
+        case 2: return ortho_stream<8, MODE>(nv, h);
+        case 3: return ortho_stream<12, MODE>(nv, h);
+        case 4: return ortho_stream<16, MODE>(nv, h);
+        case 5: return ortho_stream<20, MODE>(nv, h);
+        case 6: return ortho_stream<24, MODE>(nv, h);
+        case 7: return ortho_stream<28, MODE>(nv, h);
+        case 8: return ortho_stream<32, MODE>(nv, h);
+        case 9:
+        case 10: return ortho_stream<40, MODE>(nv, h);
+        case 11:
+        case 12: return ortho_stream<48, MODE>(nv, h);
+        case 13:
+        case 14: return ortho_stream<56, MODE>(nv, h);
+        default: return ortho_stream<64, MODE>(nv, h);
+      }
     }
-    check();
   }
 
   // Arnoldi step j of FGMRES (predicated on inner status)
@@ -1794,14 +1874,16 @@ struct Seq {
     const char* vj = (const char*)w.Vb + (size_t)j * vecb;
     char* wj1 = (char*)w.Vb + (size_t)(j + 1) * vecb;
     const void* zin = vj;
-    if (w.pc == FIT_PC_JACOBI || w.pc == FIT_PC_EPS) {
-      k_fg_precond_diag<T><<<vgrid(), 256, 0, s>>>((const V*)w.Vb, (V*)w.Zb, j, (const V*)w.dinv, w.sys, w.p);
-      check();
-      zin = (const char*)w.Zb + (size_t)j * vecb;
-    } else if (w.pc == FIT_PC_UNET && ((j + 1) % w.p.pc_every) != 0) {
-      // every other step of the cycle: the Jacobi term
-      k_fg_precond_diag<T><<<vgrid(), 256, 0, s>>>((const V*)w.Vb, (V*)w.Zb, j, (const V*)w.dinv, w.sys, w.p);
-      check();
+    // step i takes the diagonal direction z_i = D^-1 v_i (with the learned preconditioner: every step but
+    // the network's)
+    auto diag_step = [&](int i) {
+      return w.pc == FIT_PC_JACOBI || w.pc == FIT_PC_EPS || (w.pc == FIT_PC_UNET && ((i + 1) % w.p.pc_every) != 0);
+    };
+    if (diag_step(j)) {
+      if (j == 0) {  // later steps' z is written with v by k_fg_scale
+        k_fg_precond_diag<T><<<vgrid(), 256, 0, s>>>((const V*)w.Vb, (V*)w.Zb, j, (const V*)w.dinv, w.sys, w.p);
+        check();
+      }
       zin = (const char*)w.Zb + (size_t)j * vecb;
     } else if (w.pc == FIT_PC_UNET) {
       // The network's direction: z_j = U(v_i) / sqrt(n_e) + 1e-3 D^-1 v_j with i = j + 1 - pc_every and
@@ -1829,18 +1911,17 @@ struct Seq {
     ortho<T, 0>(j, nullptr);
     ortho<T, 1>(j, w.h1);
     ortho<T, 2>(j, w.h2);
-    k_fg_scale<T><<<vgrid(), 256, 0, s>>>((V*)w.Vb, j, w.sys, w.p);
+    V* zn = j + 1 < w.m && diag_step(j + 1) ? (V*)((char*)w.Zb + (size_t)(j + 1) * vecb) : nullptr;
+    k_fg_scale<T><<<vgrid(), 256, 0, s>>>((V*)w.Vb, j, zn, (const V*)w.dinv, w.sys, w.p);
     check();
   }
 
   template <typename T>
   void fg_finish() {
     using V = typename cplx<T>::t;
-    k_fg_solve<<<(w.p.B + 127) / 128, 128, 0, s>>>(w.H, w.G, w.Y, w.sys, w.p);
+    k_fg_solve<<<w.p.B, 32, 0, s>>>(w.H, w.G, w.Y, w.sys, w.p);
     check();
-    if (w.m <= 16) k_fg_combine<T, 16><<<vgrid(), 256, 0, s>>>((const V*)w.Zb, (V*)w.d, w.Y, w.sys, w.p);
-    else if (w.m <= 32) k_fg_combine<T, 32><<<vgrid(), 256, 0, s>>>((const V*)w.Zb, (V*)w.d, w.Y, w.sys, w.p);
-    else k_fg_combine<T, 64><<<vgrid(), 256, 0, s>>>((const V*)w.Zb, (V*)w.d, w.Y, w.sys, w.p);
+    k_fg_combine<T><<<vgrid(), 256, 0, s>>>((const V*)w.Zb, (V*)w.d, w.Y, w.sys, w.p);
     check();
   }
 
@@ -1867,8 +1948,6 @@ struct Seq {
     }
   }
 
-  int* mirror_inner = nullptr;  // per-system status words for the apply's predicate
-  int* mirror_outer = nullptr;
   void cond(int which, int guard_max, cudaGraphConditionalHandle h, int use_handle) {
     k_cond<<<1, 256, 0, s>>>(w.sys, w.ctl, w.p, which, guard_max, h, use_handle, mirror_inner, mirror_outer);
     check();
@@ -2052,7 +2131,6 @@ fit_status run_batch(Work& w, const double2* rhs, double2* x, cudaStream_t s, in
     } else {
       for (int j = 0; j < w.m; ++j) {
         q.fg_step<T>(j, st_inner);
-        mirror(s_outer);
       }
       q.fg_finish<T>();
     }
