@@ -78,7 +78,7 @@ __global__ void assemble_kernel(const double* __restrict__ dx, const double* __r
   };
   long long cp = i + (long long)nxp * (j + (long long)ny * k);
   double eps[3], kap[3];
-  uint8_t m = 0;
+  uint8_t m = FIT_MASK_CELL;
   // x-edge: cells (i, j-1..j, k-1..k)
   {
     double se = 0, sk = 0;
@@ -213,6 +213,21 @@ fit_status fit_take_device_error(fit_grid* g) {
   fit_set_error(code == 2 ? "a kernel of this grid stopped early: the abort word was set"
                           : "a bounded wait in a kernel of this grid ran out; its output is incomplete");
   return FIT_ETIMEOUT;
+}
+
+// the batch's frequencies into the handle's device buffer (grown on demand, counted in the budget)
+fit_status fit_stage_omega(fit_grid* g, int nbatch, const double* omega, cudaStream_t s) {
+  if (nbatch > g->omega_cap) {
+    if (g->omega_dev) fit_dev_free(g, g->omega_dev, g->omega_cap * sizeof(double));
+    g->omega_dev = nullptr;
+    g->omega_cap = 0;
+    int cap = std::max(nbatch, 64);
+    fit_status st = fit_dev_alloc(g, (void**)&g->omega_dev, cap * sizeof(double));
+    if (st != FIT_OK) return st;
+    g->omega_cap = cap;
+  }
+  FIT_CHECK_CUDA(cudaMemcpyAsync(g->omega_dev, omega, nbatch * sizeof(double), cudaMemcpyHostToDevice, s));
+  return FIT_OK;
 }
 
 extern "C" {
@@ -375,7 +390,7 @@ fit_status fit_set_material_matrices(fit_grid* g, const double* m_eps, const dou
       for (int i = 0; i < g->nx; ++i) {
         size_t c = i + (size_t)g->nx * (j + (size_t)g->ny * k);
         size_t cp = i + (size_t)g->nxp * (j + (size_t)g->ny * k);
-        uint8_t m = 0;
+        uint8_t m = FIT_MASK_CELL;
         for (int w = 0; w < 3; ++w) {
           nu[3 * cp + w] = m_nu[3 * c + w];
           ek[6 * cp + w] = m_eps[3 * c + w];
@@ -413,21 +428,6 @@ fit_status fit_grid_info(const fit_grid* g, long long* out6) {
   return FIT_OK;
 }
 
-// the batch's frequencies into the handle's device buffer (grown on demand, counted in the budget)
-static fit_status stage_omega(fit_grid* g, int nbatch, const double* omega, cudaStream_t s) {
-  if (nbatch > g->omega_cap) {
-    if (g->omega_dev) fit_dev_free(g, g->omega_dev, g->omega_cap * sizeof(double));
-    g->omega_dev = nullptr;
-    g->omega_cap = 0;
-    int cap = std::max(nbatch, 64);
-    fit_status st = fit_dev_alloc(g, (void**)&g->omega_dev, cap * sizeof(double));
-    if (st != FIT_OK) return st;
-    g->omega_cap = cap;
-  }
-  FIT_CHECK_CUDA(cudaMemcpyAsync(g->omega_dev, omega, nbatch * sizeof(double), cudaMemcpyHostToDevice, s));
-  return FIT_OK;
-}
-
 fit_status fit_apply(fit_grid* g, int nbatch, const double* omega, const void* x, void* y, fit_prec prec,
                      void* stream) {
   FIT_REQUIRE(g && omega && x && y, "fit_apply: null argument");
@@ -443,9 +443,13 @@ fit_status fit_apply(fit_grid* g, int nbatch, const double* omega, const void* x
   if (fit_check_abort(g, "fit_apply") != FIT_OK) return FIT_ETIMEOUT;
   FIT_CHECK_CUDA(cudaSetDevice(g->device));
   cudaStream_t s = (cudaStream_t)stream;
-  fit_status st = stage_omega(g, nbatch, omega, s);
-  if (st != FIT_OK) return st;
   double out_scale = prec == FIT_C64 ? 1.0 / g->coef_scale : 1.0;
+  // A small batch's frequencies travel as kernel arguments: a copy of 8 bytes in front of every apply cost the
+  // host more than the launch and stood between the kernels of consecutive applies on the device.
+  if (nbatch <= FIT_OMEGA_ARGS)
+    return fit_launch_apply(g, nbatch, fit_omega::of_host(omega), x, y, prec, out_scale, s);
+  fit_status st = fit_stage_omega(g, nbatch, omega, s);
+  if (st != FIT_OK) return st;
   return fit_launch_apply(g, nbatch, g->omega_dev, x, y, prec, out_scale, s);
 }
 
@@ -491,7 +495,7 @@ fit_status fit_apply_sym(fit_grid* g, int nbatch, const double* omega, const voi
   if (fit_check_abort(g, "fit_apply_sym") != FIT_OK) return FIT_ETIMEOUT;
   FIT_CHECK_CUDA(cudaSetDevice(g->device));
   cudaStream_t s = (cudaStream_t)stream;
-  fit_status st = stage_omega(g, nbatch, omega, s);
+  fit_status st = fit_stage_omega(g, nbatch, omega, s);
   if (st != FIT_OK) return st;
   return fit_launch_apply_sym(g, nbatch, g->omega_dev, x, y, prec, s);
 }

@@ -20,6 +20,9 @@
 // Row pitch (in cells) of the library's internal per-cell arrays is a multiple of this, so that
 // every row starts on a 16-byte boundary for the bulk tensor copies (TMA) of the fused kernel.
 #define FIT_PITCH_ALIGN 16
+// set in the mask byte of every cell of the grid, clear in the row padding (and in the zero fill of a copy
+// that reaches past the grid)
+#define FIT_MASK_CELL 8
 
 struct fit_grid {
   int nx = 0, ny = 0, nz = 0;
@@ -36,7 +39,7 @@ struct fit_grid {
   double* ek64 = nullptr;  // [ncellp*6] M_eps (x,y,z) then M_kappa (x,y,z) edge values (SI)
   float* nu32 = nullptr;   // [ncellp*3] coef_scale * M_nu
   float* ek32 = nullptr;   // [ncellp*6] coef_scale * (M_eps, M_kappa)
-  uint8_t* mask = nullptr; // [ncellp] bit w set = w-edge of the cell is masked (PEC/wall)
+  uint8_t* mask = nullptr; // [ncellp] bit w set = w-edge of the cell is masked (PEC/wall); FIT_MASK_CELL
   double coef_scale = 1.0; // c64 coefficients are coef_scale * SI values (1 / max M_nu)
   bool has_materials = false;
   bool eps_positive = false;  // M_eps > 0 and finite on every unmasked edge (the symmetrised form divides by it)
@@ -140,16 +143,34 @@ struct fit_epi {
   long long nslots = 0;  // set by the launcher: partial slots per system this launch writes
 };
 
-// Launch the operator apply: y_b = out_scale * A(omega_b) x_b (+ epilogue).  omega_dev is a
-// device array of nbatch angular frequencies.  x/y are float2 (FIT_C64) or double2 (FIT_C128).
-fit_status fit_launch_apply(fit_grid* g, int nbatch, const double* omega_dev, const void* x, void* y,
+// A batch's angular frequencies: a device array, or (up to FIT_OMEGA_ARGS of them) a host array whose values
+// travel as kernel arguments.
+#define FIT_OMEGA_ARGS 16
+struct fit_omega {
+  const double* dev = nullptr;
+  const double* host = nullptr;
+  fit_omega(const double* device_array) : dev(device_array) {}
+  static fit_omega of_host(const double* h) {
+    fit_omega o(nullptr);
+    o.host = h;
+    return o;
+  }
+};
+// copies the batch's frequencies into the handle's device buffer g->omega_dev (grown on demand)
+fit_status fit_stage_omega(fit_grid* g, int nbatch, const double* omega, cudaStream_t s);
+fit_status fit_launch_apply_generic(fit_grid* g, int nbatch, const double* omega_dev, const void* x, void* y,
+                                    fit_prec prec, double out_scale, cudaStream_t s, fit_epi* epi);
+
+// Launch the operator apply: y_b = out_scale * A(omega_b) x_b (+ epilogue).  x/y are float2 (FIT_C64) or
+// double2 (FIT_C128).
+fit_status fit_launch_apply(fit_grid* g, int nbatch, const fit_omega& omega, const void* x, void* y,
                             fit_prec prec, double out_scale, cudaStream_t stream, fit_epi* epi = nullptr);
 // the symmetrised operator of Eq. e2s (generic kernel), omega already on the device
 fit_status fit_launch_apply_sym(fit_grid* g, int nbatch, const double* omega_dev, const void* x, void* y,
                                 fit_prec prec, cudaStream_t s);
 // Time the apply variants for (nbatch, prec) on the given buffers and cache the fastest; no-op if
 // already tuned.  Must not be called while the stream is being captured.
-fit_status fit_tune_apply(fit_grid* g, int nbatch, const double* omega_dev, const void* x, void* y, fit_prec prec,
+fit_status fit_tune_apply(fit_grid* g, int nbatch, const fit_omega& omega, const void* x, void* y, fit_prec prec,
                           cudaStream_t s);
 // The cached choice: out7 = {choice (-1 generic, -2 untuned, >= 0 fused variant), TX, TY, TZ,
 // ring stages, warp-specialised (0/1), L2 prefetch distance in planes}.

@@ -45,7 +45,7 @@ fit_status noalloc_scratch(int device, double** out) {
 }  // namespace
 
 // launch without the autotuner (defined with the fused kernels)
-fit_status fit_launch_apply_fixed(fit_grid* g, int nbatch, const double* omega_dev, const void* x, void* y,
+fit_status fit_launch_apply_fixed(fit_grid* g, int nbatch, const fit_omega& omega, const void* x, void* y,
                                   fit_prec prec, double out_scale, cudaStream_t s);
 
 extern "C" fit_status fit_apply_noalloc(fit_grid* g, int nbatch, const double* omega, const void* x, void* y,
