@@ -58,6 +58,7 @@ struct Sys {
   int rin_min_it;      // iteration at which it was reached
   int mr;              // 1: the step length amr of this refinement step is still to be applied
   int replay;          // > 0: the last inner solve failed; stop the next one at this iteration
+  int dpend;           // COCG: this iteration's d += alpha p is still to be done (with the p update)
   double2 amr;         // minimal-residual step length along this step's correction
 };
 
@@ -82,6 +83,9 @@ struct P {
   int stall;         // inner solve stops after this many iterations without a new minimum
   int precond;       // right preconditioner of the inner solve (FIT_PC_*)
   int pc_every;      // FIT_PC_UNET: Arnoldi steps j with (j + 1) % pc_every == 0 take the network's direction
+  double aim;        // the last inner solve aims at this fraction of the outer tolerance
+  int trip;          // single-vector loops: iterations per pass of the inner loop (per loop test)
+  int* mirror;       // per-system inner status words that the apply's predicate reads
   const volatile int* abort;  // the grid's abort word (pinned host memory), polled by the loop conditions
   int* err;                   // the grid's error word: set to 2 when the abort word ends the loops
 };
@@ -105,39 +109,58 @@ template <> __device__ inline double2 mkc<double>(double re, double im) { return
 // Fixed-order reduction of the per-block partials of one system, then a scalar operation.
 // ------------------------------------------------------------------------------------------------
 // All 256 threads of the block call it; thread 0 receives out[0..NQ-1] = sum over the nslots
-// partials pb[s * stride + q] in a fixed order (threads take slots t, t + 256, ..., then a tree).
+// partials pb[s * stride + q] in a fixed order: 8 / NQ warps per value, their lanes taking every
+// (32 * 8 / NQ)-th slot, a shuffle tree, then the warps in order.  (GB300 adds two FP64 numbers per clock and
+// SM: a tree over 256 threads for every value spent more on its upper levels than on the slots.)
 // The partials are read through L2 (another block of the same kernel may just have written them).
 template <int NQ>
 __device__ inline void reduce_slots(const double* pb, long long nslots, int stride, double* out) {
-  __shared__ double red[256][NQ];
-  double acc[NQ];
+  constexpr int WPQ = 8 / NQ;  // warps per value
+  __shared__ double red[NQ][WPQ];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp / WPQ, part = warp % WPQ;
+  if (q < NQ) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (long long s = part * 32 + lane; s < nslots; s += 32 * WPQ) acc += __ldcg(pb + s * stride + q);
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-  for (long long s = threadIdx.x; s < nslots; s += 256)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) acc[q] += __ldcg(pb + s * stride + q);
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) red[threadIdx.x][q] = acc[q];
-  __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if ((int)threadIdx.x < h)
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) red[threadIdx.x][q] += red[threadIdx.x + h][q];
-    __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) red[q][part] = acc;
   }
+  __syncthreads();
   if (threadIdx.x == 0)
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) out[q] = red[0][q];
+    for (int k = 0; k < NQ; ++k) {
+      double t = red[k][0];
+#pragma unroll
+      for (int w = 1; w < WPQ; ++w) t += red[k][w];
+      out[k] = t;
+    }
+}
+
+// Programmatic launch (see launch_pdl): a one-block kernel may become resident while its predecessor
+// finishes; it waits here before it touches memory.  The vector passes are launched plainly: blocks that become
+// resident early take up the free slots of some SMs, and the pass then ends with those SMs behind (COCG at
+// 128^3: 132 against 126 us per iteration, 4 complex128 systems of 48x40x32: 165 against 141).
+__device__ inline void pdl_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int NQ, class Op>
 __global__ void __launch_bounds__(256) fin_kernel(const double* __restrict__ part, long long nslots, int stride,
                                                   Sys* sys, P p, Op op) {
   const int b = blockIdx.x;
-  if (!op.active(sys[b])) return;
+  pdl_start();
+  if (!op.active(sys[b])) {
+    if (threadIdx.x == 0) op.idle(sys[b]);
+    return;
+  }
   double s[NQ];
   reduce_slots<NQ>(part + (long long)b * nslots * stride, nslots, stride, s);
-  if (threadIdx.x == 0) op.apply(sys[b], s, p, b);
+  if (threadIdx.x == 0) {
+    op.apply(sys[b], s, p, b);
+    p.mirror[b] = sys[b].inner_status;
+  }
 }
 
 // The last block of a vector kernel to finish (per system) reduces the partial sums of all blocks and
@@ -155,15 +178,21 @@ __device__ inline void last_block_fin(const double* part, unsigned* cnt, Sys* sy
   if (!last) return;
   __threadfence();
   double s[NQ];
-  reduce_slots<NQ>(part + (long long)b * p.nblk * p.pstride, p.nblk, p.pstride, s);
+  reduce_slots<NQ>(part + (long long)b * gridDim.x * p.pstride, gridDim.x, p.pstride, s);
   if (threadIdx.x == 0) {
     op.apply(sys[b], s, p, b);
+    p.mirror[b] = sys[b].inner_status;
     cnt[b] = 0u;
   }
 }
 
+// what an operation does for a system it is not active for
+struct OpBase {
+  __device__ void idle(Sys&) const {}
+};
+
 // ---- outer-loop operations --------------------------------------------------------------------
-struct OpOuterInit {  // q2 = ||b||^2
+struct OpOuterInit : OpBase {  // q2 = ||b||^2
   __device__ bool active(const Sys&) const { return true; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     s.bnorm2 = q[2];
@@ -190,7 +219,7 @@ struct OpOuterInit {  // q2 = ||b||^2
 // (linear in the step, so again b - A x exactly up to rounding), whose norm never exceeds that of
 // r0 or r1: a correction that would raise the residual is shortened instead, down to none.
 // q0 = ||r0||^2, q1, q2 = Re, Im <r1, r0>, q3 = ||r1||^2.
-struct OpOuter {
+struct OpOuter : OpBase {
   __device__ bool active(const Sys& s) const { return s.outer_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     const double a = q[0], c = q[3];
@@ -226,7 +255,7 @@ struct OpOuter {
 };
 
 // inner start: q0 = ||r~||^2 (for BiCGStab rho = <r^, r> = ||r~||^2)
-struct OpInnerStart {
+struct OpInnerStart : OpBase {
   __device__ bool active(const Sys&) const { return true; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     if (s.outer_status != SYS_RUN) { s.inner_status = SYS_CONV; return; }
@@ -243,7 +272,7 @@ struct OpInnerStart {
     s.rin_min_it = 0;
     s.corr = p.s_in * s.rscale;
     // relative target of this inner solve: no tighter than needed for the outer tolerance
-    double need = 0.5 * sqrt(s.tol2) / s.rscale;
+    double need = p.aim * sqrt(s.tol2) / s.rscale;
     double it = p.mixed ? fmax(p.inner_tol, need) : fmax(need, 1e-15);
     s.inner_tol2 = it * it * q[0];
     s.max_inner = max(1, p.max_iter - s.iters);
@@ -262,7 +291,7 @@ struct OpInnerStart {
 // form (u, v) = sum_i u_i v_i in place of the inner product, right/left-symmetric Jacobi
 // preconditioner z = D^-1 r.  Per iteration: q = A p, alpha = rho / (p, q), d += alpha p,
 // r -= alpha q, rho' = (r, D^-1 r), beta = rho' / rho, p = D^-1 r + beta p.
-struct OpCocgStart {  // q0,q1 = (r~, D^-1 r~), q2 = ||r~||^2
+struct OpCocgStart : OpBase {  // q0,q1 = (r~, D^-1 r~), q2 = ||r~||^2
   __device__ bool active(const Sys&) const { return true; }
   __device__ void apply(Sys& s, const double* q, const P& p, int b) const {
     const double qq[3] = {q[2], 0.0, 0.0};
@@ -272,17 +301,20 @@ struct OpCocgStart {  // q0,q1 = (r~, D^-1 r~), q2 = ||r~||^2
   }
 };
 
-struct OpCocgAlpha {  // q0,q1 = (p, A p)
+struct OpCocgAlpha : OpBase {  // q0,q1 = (p, A p)
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
+  __device__ void idle(Sys& s) const { s.dpend = 0; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     double2 sig = make_double2(q[0], q[1]);
+    s.dpend = 0;
     if (!cfinite(sig)) { s.inner_status = SYS_NAN; return; }
     if (sqrt(cabs2(sig)) < p.tiny) { s.inner_status = SYS_BREAK; return; }
     s.alpha = cdiv(s.rho, sig);
+    s.dpend = 1;
   }
 };
 
-struct OpCocgRho {  // q0,q1 = (r, D^-1 r), q2 = ||r||^2
+struct OpCocgRho : OpBase {  // q0,q1 = (r, D^-1 r), q2 = ||r||^2
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     double2 rn = make_double2(q[0], q[1]);
@@ -316,7 +348,7 @@ struct OpCocgRho {  // q0,q1 = (r, D^-1 r), q2 = ||r||^2
 //   w = A z;  rho' = (z, w);  beta = rho' / rho (0 on the first);  p = z + beta p;  q = w + beta q;
 //   alpha = rho' / (q, M q);  d += alpha p;  r -= alpha q;  z = M r
 // so that q = A p throughout and each iteration costs one apply.
-struct OpCocrStart {  // q2 = ||r~||^2
+struct OpCocrStart : OpBase {  // q2 = ||r~||^2
   __device__ bool active(const Sys&) const { return true; }
   __device__ void apply(Sys& s, const double* q, const P& p, int b) const {
     const double qq[3] = {q[2], 0.0, 0.0};
@@ -325,7 +357,7 @@ struct OpCocrStart {  // q2 = ||r~||^2
   }
 };
 
-struct OpCocrBeta {  // q0,q1 = (z, A z)
+struct OpCocrBeta : OpBase {  // q0,q1 = (z, A z)
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     const double2 rn = make_double2(q[0], q[1]);
@@ -336,7 +368,7 @@ struct OpCocrBeta {  // q0,q1 = (z, A z)
   }
 };
 
-struct OpCocrAlpha {  // q0,q1 = (q, M q)
+struct OpCocrAlpha : OpBase {  // q0,q1 = (q, M q)
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     const double2 sig = make_double2(q[0], q[1]);
@@ -346,7 +378,7 @@ struct OpCocrAlpha {  // q0,q1 = (q, M q)
   }
 };
 
-struct OpCocrRes {  // q2 = ||r||^2 after the update
+struct OpCocrRes : OpBase {  // q2 = ||r||^2 after the update
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     const double rr = q[2];
@@ -367,7 +399,7 @@ struct OpCocrRes {  // q2 = ||r||^2 after the update
 };
 
 // ---- BiCGStab operations -----------------------------------------------------------------------
-struct OpAlpha {  // q0,q1 = <r^, v>
+struct OpAlpha : OpBase {  // q0,q1 = <r^, v>
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     double2 sig = make_double2(q[0], q[1]);
@@ -377,7 +409,7 @@ struct OpAlpha {  // q0,q1 = <r^, v>
   }
 };
 
-struct OpOmega {  // q0,q1 = <t, s>, q2 = <t, t>
+struct OpOmega : OpBase {  // q0,q1 = <t, s>, q2 = <t, t>
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P&, int) const {
     double tt = q[2];
@@ -386,7 +418,7 @@ struct OpOmega {  // q0,q1 = <t, s>, q2 = <t, t>
   }
 };
 
-struct OpRho {  // q0,q1 = <r^, r_new>, q2 = ||r_new||^2
+struct OpRho : OpBase {  // q0,q1 = <r^, r_new>, q2 = ||r_new||^2
   __device__ bool active(const Sys& s) const { return s.inner_status == SYS_RUN; }
   __device__ void apply(Sys& s, const double* q, const P& p, int) const {
     double2 rn = make_double2(q[0], q[1]);
@@ -419,7 +451,15 @@ struct OpRho {  // q0,q1 = <r^, r_new>, q2 = ||r_new||^2
 // e = k*256 + t + n*nblk*256 (fixed assignment, so partial sums are reproducible).
 // ------------------------------------------------------------------------------------------------
 #define VEC_LOOP(p) for (long long e = blockIdx.x * 256LL + threadIdx.x; e < (p).ne; e += (long long)gridDim.x * 256)
-#define PSLOT(p, b) ((((long long)(b) * (p).nblk + blockIdx.x)) * (p).pstride)
+#define PSLOT(p, b) ((((long long)(b) * gridDim.x + blockIdx.x)) * (p).pstride)
+
+// The passes of an iteration take VU elements per thread and trip, all loads before any use: half the
+// blocks of a one-element pass have the same bytes in flight, and half as many partial sums to add up in FP64.
+constexpr int VU = 2;
+#define VEC_TRIP(p) \
+  for (long long e0 = blockIdx.x * 256LL + threadIdx.x, es = (long long)gridDim.x * 256; e0 < (p).ne; e0 += VU * es)
+#define VEC_EACH(p) \
+  _Pragma("unroll") for (int u = 0; u < VU; ++u) if (const long long e = e0 + u * es; e < (p).ne)
 
 __global__ void __launch_bounds__(256) k_outer_init(const double2* __restrict__ rhs, double2* __restrict__ x,
                                                     double2* __restrict__ r, double* part, P p) {
@@ -567,34 +607,44 @@ __global__ void __launch_bounds__(256) k_fg_precond_diag(const typename cplx<T>:
   VEC_LOOP(p) { Zb[(long long)j * vs + off + e] = cmulv(dinv[off + e], Vb[(long long)j * vs + off + e]); }
 }
 
-// BiCGStab: d += alpha p + omega s; r = s - omega t; q0,q1 = <r^, r>, q2 = ||r||^2
+// BiCGStab: d += alpha p + omega s; r = s - omega t; q0,q1 = <r^, r>, q2 = ||r||^2; the last block applies OpRho
 template <typename T>
 __global__ void __launch_bounds__(256) k_bicg_xr(typename cplx<T>::t* d, const typename cplx<T>::t* __restrict__ pv,
                                                  typename cplx<T>::t* r, const typename cplx<T>::t* __restrict__ t,
                                                  const typename cplx<T>::t* __restrict__ shat,
-                                                 const typename cplx<T>::t* __restrict__ rhat, const Sys* __restrict__ sys,
-                                                 double* part, P p) {
+                                                 const typename cplx<T>::t* __restrict__ rhat, Sys* sys,
+                                                 double* part, unsigned* cnt, P p) {
   using V = typename cplx<T>::t;
   const int b = blockIdx.y;
   if (sys[b].inner_status != SYS_RUN) return;
   const long long off = (long long)b * p.ne;
   const T ar = (T)sys[b].alpha.x, ai = (T)sys[b].alpha.y, orr = (T)sys[b].omega.x, oi = (T)sys[b].omega.y;
   T acc[3] = {T(0), T(0), T(0)};
-  VEC_LOOP(p) {
-    V s = r[off + e], pp = pv[off + e], tt = t[off + e], dd = d[off + e], rh = rhat[off + e];
-    const V sx = shat ? shat[off + e] : s;  // the update uses the preconditioned s
-    dd.x += (ar * pp.x - ai * pp.y) + (orr * sx.x - oi * sx.y);
-    dd.y += (ar * pp.y + ai * pp.x) + (orr * sx.y + oi * sx.x);
-    V rn;
-    rn.x = s.x - (orr * tt.x - oi * tt.y);
-    rn.y = s.y - (orr * tt.y + oi * tt.x);
-    d[off + e] = dd;
-    r[off + e] = rn;
-    acc[0] += rh.x * rn.x + rh.y * rn.y;
-    acc[1] += rh.x * rn.y - rh.y * rn.x;
-    acc[2] += rn.x * rn.x + rn.y * rn.y;
+  VEC_TRIP(p) {
+    V s[VU], pp[VU], tt[VU], dd[VU], rh[VU], sx[VU];
+    VEC_EACH(p) {
+      s[u] = r[off + e];
+      pp[u] = pv[off + e];
+      tt[u] = t[off + e];
+      dd[u] = d[off + e];
+      rh[u] = rhat[off + e];
+      sx[u] = shat ? shat[off + e] : s[u];  // the update uses the preconditioned s
+    }
+    VEC_EACH(p) {
+      dd[u].x += (ar * pp[u].x - ai * pp[u].y) + (orr * sx[u].x - oi * sx[u].y);
+      dd[u].y += (ar * pp[u].y + ai * pp[u].x) + (orr * sx[u].y + oi * sx[u].x);
+      V rn;
+      rn.x = s[u].x - (orr * tt[u].x - oi * tt[u].y);
+      rn.y = s[u].y - (orr * tt[u].y + oi * tt[u].x);
+      d[off + e] = dd[u];
+      r[off + e] = rn;
+      acc[0] += rh[u].x * rn.x + rh[u].y * rn.y;
+      acc[1] += rh[u].x * rn.y - rh[u].y * rn.x;
+      acc[2] += rn.x * rn.x + rn.y * rn.y;
+    }
   }
   fit_block_sum<T, 3>(acc, part + PSLOT(p, b));
+  last_block_fin<3>(part, cnt, sys, p, b, OpRho{});
 }
 
 // q0,q1 = <t, s>, q2 = <t, t> (BiCGStab omega with a right preconditioner)
@@ -737,53 +787,75 @@ __global__ void __launch_bounds__(256) k_cocg_start(const double2* __restrict__ 
   fit_block_sum<T, 3>(acc, part + PSLOT(p, b));
 }
 
-// COCG: d += alpha p, r -= alpha q; partials (r, D^-1 r), ||r||^2; the last block applies OpCocgRho
+// COCG: r -= alpha q; partials (r, D^-1 r), ||r||^2; the last block applies OpCocgRho.  (d += alpha p waits for
+// the p update, which reads p anyway: 88 -> 80 B per unknown for the two passes.)
 template <typename T>
-__global__ void __launch_bounds__(256) k_cocg_xr(typename cplx<T>::t* d, const typename cplx<T>::t* __restrict__ pv,
-                                                 typename cplx<T>::t* r, const typename cplx<T>::t* __restrict__ q,
-                                                 const typename cplx<T>::t* __restrict__ dinv, Sys* sys,
-                                                 double* part, unsigned* cnt, P p) {
+__global__ void __launch_bounds__(256) k_cocg_r(typename cplx<T>::t* __restrict__ r,
+                                                const typename cplx<T>::t* __restrict__ q,
+                                                const typename cplx<T>::t* __restrict__ dinv, Sys* sys, double* part,
+                                                unsigned* cnt, P p) {
   using V = typename cplx<T>::t;
   const int b = blockIdx.y;
   if (sys[b].inner_status != SYS_RUN) return;
   const long long off = (long long)b * p.ne;
   const T ar = (T)sys[b].alpha.x, ai = (T)sys[b].alpha.y;
   T acc[3] = {T(0), T(0), T(0)};
-  VEC_LOOP(p) {
-    const V pp = pv[off + e], qq = q[off + e];
-    V dd = d[off + e], rr = r[off + e];
-    dd.x += ar * pp.x - ai * pp.y;
-    dd.y += ar * pp.y + ai * pp.x;
-    rr.x -= ar * qq.x - ai * qq.y;
-    rr.y -= ar * qq.y + ai * qq.x;
-    d[off + e] = dd;
-    r[off + e] = rr;
-    const V z = dinv ? cmulv(dinv[off + e], rr) : rr;
-    acc[0] += rr.x * z.x - rr.y * z.y;
-    acc[1] += rr.x * z.y + rr.y * z.x;
-    acc[2] += rr.x * rr.x + rr.y * rr.y;
+  VEC_TRIP(p) {
+    V qq[VU], rr[VU], dd[VU];
+    VEC_EACH(p) {
+      qq[u] = q[off + e];
+      rr[u] = r[off + e];
+      if (dinv) dd[u] = dinv[off + e];
+    }
+    VEC_EACH(p) {
+      rr[u].x -= ar * qq[u].x - ai * qq[u].y;
+      rr[u].y -= ar * qq[u].y + ai * qq[u].x;
+      r[off + e] = rr[u];
+      const V z = dinv ? cmulv(dd[u], rr[u]) : rr[u];
+      acc[0] += rr[u].x * z.x - rr[u].y * z.y;
+      acc[1] += rr[u].x * z.y + rr[u].y * z.x;
+      acc[2] += rr[u].x * rr[u].x + rr[u].y * rr[u].y;
+    }
   }
   fit_block_sum<T, 3>(acc, part + PSLOT(p, b));
   last_block_fin<3>(part, cnt, sys, p, b, OpCocgRho{});
 }
 
-// COCG: p = D^-1 r + beta p
+// COCG: d += alpha p (also after the iteration that ended the inner solve), p = D^-1 r + beta p
 template <typename T>
-__global__ void __launch_bounds__(256) k_cocg_p(const typename cplx<T>::t* __restrict__ r, typename cplx<T>::t* pv,
-                                                const typename cplx<T>::t* __restrict__ dinv, const Sys* __restrict__ sys,
-                                                P p) {
+__global__ void __launch_bounds__(256) k_cocg_dp(typename cplx<T>::t* __restrict__ d,
+                                                 const typename cplx<T>::t* __restrict__ r,
+                                                 typename cplx<T>::t* __restrict__ pv,
+                                                 const typename cplx<T>::t* __restrict__ dinv,
+                                                 const Sys* __restrict__ sys, P p) {
   using V = typename cplx<T>::t;
   const int b = blockIdx.y;
-  if (sys[b].inner_status != SYS_RUN) return;
+  if (!sys[b].dpend) return;
+  const bool more = sys[b].inner_status == SYS_RUN;
   const long long off = (long long)b * p.ne;
-  const T br = (T)sys[b].beta.x, bi = (T)sys[b].beta.y;
-  VEC_LOOP(p) {
-    const V rr = r[off + e], pp = pv[off + e];
-    const V z = dinv ? cmulv(dinv[off + e], rr) : rr;
-    V o;
-    o.x = z.x + br * pp.x - bi * pp.y;
-    o.y = z.y + br * pp.y + bi * pp.x;
-    pv[off + e] = o;
+  const T ar = (T)sys[b].alpha.x, ai = (T)sys[b].alpha.y, br = (T)sys[b].beta.x, bi = (T)sys[b].beta.y;
+  VEC_TRIP(p) {
+    V dd[VU], rr[VU], pp[VU], di[VU];
+    VEC_EACH(p) {
+      pp[u] = pv[off + e];
+      dd[u] = d[off + e];
+      if (more) {
+        rr[u] = r[off + e];
+        if (dinv) di[u] = dinv[off + e];
+      }
+    }
+    VEC_EACH(p) {
+      dd[u].x += ar * pp[u].x - ai * pp[u].y;
+      dd[u].y += ar * pp[u].y + ai * pp[u].x;
+      d[off + e] = dd[u];
+      if (more) {
+        const V z = dinv ? cmulv(di[u], rr[u]) : rr[u];
+        V o;
+        o.x = z.x + br * pp[u].x - bi * pp[u].y;
+        o.y = z.y + br * pp[u].y + bi * pp[u].x;
+        pv[off + e] = o;
+      }
+    }
   }
 }
 
@@ -1449,6 +1521,7 @@ __global__ void k_nusum(const T* __restrict__ nu, int nx, int ny, int nz, int nx
 __global__ void k_cond(const Sys* __restrict__ sys, Ctl* ctl, P p, int which, int guard_max,
                        cudaGraphConditionalHandle h, int use_handle, int* mirror_inner, int* mirror_outer) {
   __shared__ int any;
+  pdl_start();
   if (threadIdx.x == 0) any = 0;
   __syncthreads();
   for (int b = threadIdx.x; b < p.B; b += blockDim.x) {
@@ -1464,7 +1537,7 @@ __global__ void k_cond(const Sys* __restrict__ sys, Ctl* ctl, P p, int which, in
     // the host's abort word ends both loops: read at every outer step and every 64th inner step (a
     // read of pinned host memory costs about a microsecond)
     bool stop = false;
-    if (p.abort && (which == 1 || (*guard & 63) == 1) && *p.abort) {
+    if (p.abort && (which == 1 || (*guard & (64 / p.trip - 1)) == 1) && *p.abort) {
       stop = true;
       atomicMax(p.err, 2);
     }
@@ -1635,6 +1708,9 @@ fit_status setup(Work& w, int B) {
   // residual norm is not monotone (A is complex symmetric, not Hermitian) and can wander above its
   // minimum for thousands of iterations before it falls again, so it gets a far longer window
   w.p.stall = (w.method == FIT_COCG || w.method == FIT_COCR) ? 20000 : 1000;
+  // (complex64 BiCGStab's recurrence residual leaves the true one by a few times its own size near the end: a
+  // lower aim costs 3% more iterations and halves the error of x)
+  w.p.aim = w.method == FIT_BICGSTAB && w.mixed ? 0.2 : 0.5;
   w.p.precond = w.pc;
   w.p.abort = g->abort_dev;
   w.p.err = g->err_dev;
@@ -1667,10 +1743,34 @@ struct Seq {
       st = FIT_ECUDA;
     }
   }
+  // launch of a kernel that begins with pdl_start: it may become resident before its predecessor in the
+  // stream has finished
+  template <typename... Params, typename... Args>
+  void launch_pdl(void (*kern)(Params...), dim3 grid, int threads, Args... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    check();
+  }
+  // grid of an iteration's vector pass: a few blocks per SM shared by the batch.  One large complex64 system
+  // wants more bytes in flight (4: 127.8, 6: 126.9, 8: 130.2 us per COCG iteration at 128^3); small batches and
+  // complex128 fewer partial sums in FP64 (8 x 40x36x28: 4: 62.0, 6: 64.3; complex128 4: 139.7, 8: 147.8).
+  dim3 igrid() const {
+    const int per_sm = w.mixed && w.p.B == 1 ? 6 : 4;
+    const long long fill = (w.p.ne + 255) / 256;
+    const long long n = std::max(1LL, (long long)per_sm * w.nsm / w.p.B);
+    return dim3((unsigned)std::max(1LL, std::min({n, fill, (long long)w.p.nblk})), w.p.B);
+  }
   template <int NQ, class Op>
   void fin(const double* part, long long nslots, int stride, Op op) {
-    fin_kernel<NQ, Op><<<w.p.B, 256, 0, s>>>(part, nslots, stride, w.sys, w.p, op);
-    check();
+    launch_pdl(fin_kernel<NQ, Op>, dim3(w.p.B), 256, part, nslots, stride, w.sys, w.p, op);
   }
   // launches the apply and returns the number of partial slots per system it writes
   long long apply(const void* xin, void* yout, int mode, const void* u, fit_prec prec, const int* status_field) {
@@ -1731,16 +1831,15 @@ struct Seq {
   }
 
   // one COCG iteration (predicated on inner status): q = A p with (p, q) from the apply's epilogue,
-  // alpha, the x/r update (its last block computes rho and beta), then p
+  // alpha, the r update (its last block computes rho and beta), then d and p
   template <typename T>
   void cocg_iter(const int* st_inner) {
     using V = typename cplx<T>::t;
     long long n1 = apply(w.pv, w.v, FIT_EPI_DOT_XY, nullptr, w.inner, st_inner);
     fin<3>(w.part_apply, n1, 4, OpCocgAlpha{});
-    k_cocg_xr<T><<<vgrid(), 256, 0, s>>>((V*)w.d, (const V*)w.pv, (V*)w.rin, (const V*)w.v, (const V*)w.dinv, w.sys,
-                                         w.part_vec, w.cnt, w.p);
+    k_cocg_r<T><<<igrid(), 256, 0, s>>>((V*)w.rin, (const V*)w.v, (const V*)w.dinv, w.sys, w.part_vec, w.cnt, w.p);
     check();
-    k_cocg_p<T><<<vgrid(), 256, 0, s>>>((const V*)w.rin, (V*)w.pv, (const V*)w.dinv, w.sys, w.p);
+    k_cocg_dp<T><<<igrid(), 256, 0, s>>>((V*)w.d, (const V*)w.rin, (V*)w.pv, (const V*)w.dinv, w.sys, w.p);
     check();
   }
 
@@ -1775,8 +1874,8 @@ struct Seq {
   void bicg_iter(const int* st_inner) {
     using V = typename cplx<T>::t;
     const bool pc = w.dinv != nullptr;
-    k_bicg_p<T><<<vgrid(), 256, 0, s>>>((const V*)w.rin, (V*)w.pv, (const V*)w.v, (const V*)w.dinv, (V*)w.phat,
-                                        w.sys, w.p);
+    k_bicg_p<T><<<vgrid(), 256, 0, s>>>((const V*)w.rin, (V*)w.pv, (const V*)w.v, (const V*)w.dinv, (V*)w.phat, w.sys,
+               w.p);
     check();
     long long n1 = apply(pc ? w.phat : w.pv, w.v, FIT_EPI_DOT_U, w.rhat, w.inner, st_inner);
     fin<3>(w.part_apply, n1, 4, OpAlpha{});
@@ -1792,10 +1891,9 @@ struct Seq {
     } else {
       fin<3>(w.part_apply, n2, 4, OpOmega{});
     }
-    k_bicg_xr<T><<<vgrid(), 256, 0, s>>>((V*)w.d, (const V*)(pc ? w.phat : w.pv), (V*)w.rin, (const V*)w.t,
-                                         (const V*)(pc ? w.shat : nullptr), (const V*)w.rhat, w.sys, w.part_vec, w.p);
+    k_bicg_xr<T><<<igrid(), 256, 0, s>>>((V*)w.d, (const V*)(pc ? w.phat : w.pv), (V*)w.rin, (const V*)w.t,
+               (const V*)(pc ? w.shat : nullptr), (const V*)w.rhat, w.sys, w.part_vec, w.cnt, w.p);
     check();
-    fin<3>(w.part_vec, w.p.nblk, w.p.pstride, OpRho{});
   }
 
   // the three CGS2 passes over V[0..j] (mode 0: dots; 1: update with h, dots; 2: update with h2, norm), each
@@ -1949,8 +2047,7 @@ struct Seq {
   }
 
   void cond(int which, int guard_max, cudaGraphConditionalHandle h, int use_handle) {
-    k_cond<<<1, 256, 0, s>>>(w.sys, w.ctl, w.p, which, guard_max, h, use_handle, mirror_inner, mirror_outer);
-    check();
+    launch_pdl(k_cond, dim3(1), 256, w.sys, w.ctl, w.p, which, guard_max, h, use_handle, mirror_inner, mirror_outer);
   }
 };
 
@@ -1972,6 +2069,8 @@ fit_status run_batch(Work& w, const double2* rhs, double2* x, cudaStream_t s, in
   fit_status st;
   if ((st = w.alloc((void**)&st_inner, w.p.B * sizeof(int))) != FIT_OK) return st;
   if ((st = w.alloc((void**)&st_outer, w.p.B * sizeof(int))) != FIT_OK) return st;
+  w.p.mirror = st_inner;
+  w.p.trip = use_graph ? 8 : 1;
   Seq q{w, rhs, x, s};
   q.mirror_inner = st_inner;
   q.mirror_outer = st_outer;
@@ -2123,7 +2222,9 @@ fit_status run_batch(Work& w, const double2* rhs, double2* x, cudaStream_t s, in
            "capture inner body");
       if (result != FIT_OK) break;
       q.s = s_inner;
-      q.loop_iter<T>(st_inner);
+      // several iterations per pass of the WHILE node: a pass costs about 6 us of its own (COCG at 128^3: 134.7
+      // us per iteration with one, 127.4 with eight), and the kernels of systems that have finished return at once
+      for (int it = 0; it < w.p.trip; ++it) q.loop_iter<T>(st_inner);
       q.cond(0, max_inner_guard, h_inner, 1);
       cudaGraph_t tmp;
       fail(cudaStreamEndCapture(s_inner, &tmp), "end inner");
