@@ -290,15 +290,38 @@ static fit_status conv3_tc(const unet::ConvArgs& a, int cin, cudaStream_t s, boo
 }
 
 // Weight gradient of a 3x3x3 conv on the tensor cores: dw (27 x cout x cin) and db accumulate (the caller
-// zeroes them); chunks of 1024 voxels per block, 27 taps.
-fit_status wgrad_launch(const unet::WgradArgs& w0, cudaStream_t s) {
-  unet::WgradArgs w = w0;
-  w.chunk = 1024;
-  const long long nv = (long long)w.nx * w.ny * w.nz;
-  const dim3 grid((unsigned)((nv + w.chunk - 1) / w.chunk), 27);
+// zeroes them).  Two blocks per SM, a third of them for each z-tap, every one with about three row
+// segments' worth of y-chunks (at least eight rows each, so that a chunk's two halo rows stay a small part).
+template <int CO, int CI, int TV>
+fit_status wgrad_launch_shape(const unet::WgradArgs& w, cudaStream_t s) {
+  auto kern = unet::conv3_wgrad_kernel<CO, CI, TV>;
+  constexpr int smem = unet::WgradShape<CO, CI>::smem(TV);
+  int dev = 0, nsm = 0;
+  FIT_CHECK_CUDA(cudaGetDevice(&dev));
+  FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int blocks = std::max(1, 2 * nsm / 3);
+  const long long rows = (long long)((w.nx + TV - 1) / TV) * w.nz;
+  const int most = std::max(1, w.ny / 8);
+  const int nyc = (int)std::min<long long>(most, std::max(1LL, (3LL * blocks + rows - 1) / rows));
+  const int ylen = (w.ny + nyc - 1) / nyc, chunks = (w.ny + ylen - 1) / ylen;
+  const long long ntask = rows * chunks;
+  if (ntask > (1LL << 30)) {
+    fit_set_error("U-Net: grid too large for the weight gradient");
+    return FIT_EINVAL;
+  }
+  const dim3 grid((unsigned)std::min<long long>(ntask, blocks), 3);
+  kern<<<grid, 256, smem, s>>>(w, ylen, chunks, (int)ntask);
+  FIT_CHECK_CUDA(cudaGetLastError());
+  return FIT_OK;
+}
+
+fit_status wgrad_launch(const unet::WgradArgs& w, cudaStream_t s) {
   const int ci = w.c1 + w.c2, co = w.cout;
+  // segments of 64 voxels, of 32 where a row has no more (half of a longer one would be padding)
 #define FIT_WG(CO_, CI_) \
-  if (co == CO_ && ci == CI_) { unet::conv3_wgrad_mma_kernel<CO_, CI_><<<grid, 256, 0, s>>>(w); return FIT_OK; }
+  if (co == CO_ && ci == CI_) \
+    return w.nx <= 32 ? wgrad_launch_shape<CO_, CI_, 32>(w, s) : wgrad_launch_shape<CO_, CI_, 64>(w, s)
   FIT_WG(16, 16);
   FIT_WG(32, 16);
   FIT_WG(32, 32);

@@ -535,20 +535,10 @@ struct WgradArgs {
   int c1, c2;      // input channels of the forward conv (split over two sources)
   int cout;
   float* dw;       // [27][cout][c1 + c2]
-  float* db;       // [cout] or null (accumulated by tap 13)
+  float* db;       // [cout] or null (summed by the blocks of the central z-tap)
   int nx, ny, nz;
-  int chunk;       // voxels per CTA
 };
 
-// On the tensor cores (mma.sync m16n8k16, bf16 x bf16 -> FP32): for one tap,
-//   dW[tap] (CO x CI) += dY^T (CO x V) X_tap (V x CI),   X_tap[v] = x[v + off(tap)] (zero outside),
-// a GEMM whose K dimension is the voxels.  A block takes one tap (blockIdx.y) and a chunk of voxels
-// (blockIdx.x), stages 64 voxels at a time as [voxel][channel] rows of dY and of the shifted X (rows
-// padded by 8 channels, so that the 8 rows an ldmatrix reads start in distinct banks) and reads them as
-// transposed fragments (ldmatrix .trans): the MMA's A operand is dY^T, its B operand X_tap.  The 4 K-steps
-// of 16 voxels times the (CO/16) x (CI/8) output tiles are spread over the 8 warps, each warp keeping
-// FP32 accumulators for its tiles across all of the block's voxels; the block's partial dW is added with
-// FP32 atomics, and the centre tap's blocks also sum dY for db.
 // ------------------------------------------------------------------------------------------------
 __device__ inline void ldsm_x4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -559,83 +549,178 @@ __device__ inline void ldsm_x2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
 }
 
+// One block works on row segments of TV voxels along x and marches along y: per step it brings in one row of
+// dY and one of X (in the plane z + dz - 1, dz = blockIdx.y), with the X rows y-1, y, y+1 and one voxel of halo at
+// either end in shared memory, and adds the nine in-plane taps' products, so that a voxel is read three times
+// (once per dz) instead of 27 times.  dW[tap] (CO x CI) += dY^T (CO x TV) X_tap (TV x CI) as m16n8k16 MMAs whose
+// fragments come by transposed ldmatrix; a tap's shift along x is a row offset of the fragment.  The nine
+// taps' accumulators stay in registers over all of the block's segments: the eight warps are WT groups of
+// (16 output channel) x (8 NCB input channel) columns times WK shares of the segment's voxels.  Rows arrive
+// by cp.async two steps ahead (zero fill outside the grid).  What bounds it: the MMAs and their ldmatrix
+// traffic (one B fragment per MMA for NCB = 1); the final adds are vector reductions to L2, one set per
+// block.  32 -> 16 at 64^3: 221 us with a block per (1024 voxels, tap), each re-reading X and dY and
+// dividing out every voxel's coordinates.
 template <int CO, int CI>
-__global__ void __launch_bounds__(256) conv3_wgrad_mma_kernel(WgradArgs a) {
-  constexpr int TV = 64, RSO = CO + 8, RSI = CI + 8;
-  constexpr int MT = CO / 16, NT = CI / 8, TILES = MT * NT;
-  constexpr int NACC = TILES >= 8 ? TILES / 8 : 1;  // output tiles per warp
-  static_assert(CO % 16 == 0 && CI % 8 == 0 && (TILES % 8 == 0 || 8 % TILES == 0), "wgrad tile shape");
-  __shared__ __align__(16) bf16 sdy[TV * RSO];
-  __shared__ __align__(16) bf16 sx[TV * RSI];
+struct WgradShape {
+  static constexpr int MT = CO / 16, NT = CI / 8, COMBOS = MT * NT;
+  static constexpr int WT = COMBOS >= 16 ? 8 : (COMBOS >= 4 ? 4 : 2), WK = 8 / WT;
+  static constexpr int NCB = COMBOS / WT;  // 8-channel columns per warp, all of one 16-row group
+  static constexpr int RSO = CO + 8, RSI = CI + 8;  // padded row strides (conflict-free ldmatrix)
+  static constexpr int XR = 8, YR = 4;              // rings: rows of X and of dY
+  static constexpr int stage_bytes(int TV) { return (XR * (TV + 2) * RSI + YR * TV * RSO) * 2; }
+  static constexpr int smem(int TV) {
+    const int sum = 9 * CO * CI * 4;
+    return WK > 1 && sum > stage_bytes(TV) ? sum : stage_bytes(TV);
+  }
+};
+
+template <int CO, int CI, int TV>
+__global__ void __launch_bounds__(256) conv3_wgrad_kernel(WgradArgs a, int ylen, int nyc, int ntask) {
+  using SH = WgradShape<CO, CI>;
+  constexpr int RSO = SH::RSO, RSI = SH::RSI, NCB = SH::NCB, WK = SH::WK, XR = SH::XR, YR = SH::YR;
+  constexpr int KS = TV / 16;
+  static_assert(CO % 16 == 0 && CI % 16 == 0 && SH::NT % NCB == 0 && TV % 16 == 0, "wgrad tile shape");
+  extern __shared__ __align__(16) unsigned char wg_smem[];
+  bf16* sx = (bf16*)wg_smem;                 // [XR][TV + 2][RSI]
+  bf16* sdy = sx + XR * (TV + 2) * RSI;      // [YR][TV][RSO]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tap = blockIdx.y;
-  const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-  const long long nvox = (long long)a.nx * a.ny * a.nz;
-  const long long v0 = (long long)blockIdx.x * a.chunk;
-  const long long v1 = min(nvox, v0 + a.chunk);
-  float acc[NACC][4];
-#pragma unroll
-  for (int j = 0; j < NACC; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-  float dbs = 0.f;
+  const int dz = (int)blockIdx.y;
+  const int wt = warp / WK, wk = warp % WK;
+  const int mt = (wt * NCB) / SH::NT, nt0 = (wt * NCB) % SH::NT;
   const int q = lane >> 3, r = lane & 7;  // ldmatrix: which 8x8 matrix this lane addresses, and its row
-  for (long long vb = v0; vb < v1; vb += TV) {
-    __syncthreads();  // the previous tile's fragments are read
-    for (int e = tid; e < TV * (CO / 8); e += 256) {  // dY rows, 16-byte vectors
-      const int vi = e / (CO / 8), c8 = e % (CO / 8);
-      const long long v = vb + vi;
-      uint4 val = make_uint4(0u, 0u, 0u, 0u);
-      if (v < v1) val = *reinterpret_cast<const uint4*>(a.dy + v * CO + c8 * 8);
-      *reinterpret_cast<uint4*>(sdy + vi * RSO + c8 * 8) = val;
-    }
-    for (int e = tid; e < TV * (CI / 8); e += 256) {  // X rows shifted by the tap
-      const int vi = e / (CI / 8), c8 = e % (CI / 8);
-      const long long v = vb + vi;
-      uint4 val = make_uint4(0u, 0u, 0u, 0u);
-      if (v < v1) {
-        const int x = (int)(v % a.nx), y = (int)((v / a.nx) % a.ny), z = (int)(v / ((long long)a.nx * a.ny));
-        const int xs = x + dx, ys = y + dy, zs = z + dz;
-        if (xs >= 0 && ys >= 0 && zs >= 0 && xs < a.nx && ys < a.ny && zs < a.nz) {
-          const long long vs = xs + (long long)a.nx * (ys + (long long)a.ny * zs);
-          const int c = c8 * 8;
-          val = c < a.c1 ? *reinterpret_cast<const uint4*>(a.x1 + vs * a.c1 + c)
-                         : *reinterpret_cast<const uint4*>(a.x2 + vs * a.c2 + (c - a.c1));
+  const int nseg = (a.nx + TV - 1) / TV;
+  float acc[9][NCB][4];
+#pragma unroll
+  for (int t = 0; t < 9; ++t)
+#pragma unroll
+    for (int n = 0; n < NCB; ++n)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[t][n][c] = 0.f;
+  float dbs = 0.f;  // dz = 1: this thread's share of db[tid % CO]
+  for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+    const int xs = (task % nseg) * TV, yc = (task / nseg) % nyc, z = task / (nseg * nyc);
+    const int zx = z + dz - 1;
+    if (zx < 0 || zx >= a.nz) continue;  // (dz = 1 never is: db misses nothing)
+    const int y0 = yc * ylen, y1 = min(a.ny, y0 + ylen);
+    auto load_x = [&](int y) {  // row y of the plane zx, voxels xs-1 .. xs+TV
+      bf16* dst = sx + ((y + 1) & (XR - 1)) * (TV + 2) * RSI;
+      const bool yin = y >= 0 && y < a.ny;
+      const long long row = (long long)a.nx * (y + (long long)a.ny * zx);
+      for (int e = tid; e < (TV + 2) * (CI / 8); e += 256) {
+        const int v = e / (CI / 8), c = (e % (CI / 8)) * 8, gx = xs - 1 + v;
+        const bool in = yin && gx >= 0 && gx < a.nx;
+        const bf16* src = a.dy;  // a valid address even when nothing is read
+        if (in) src = c < a.c1 ? a.x1 + (row + gx) * a.c1 + c : a.x2 + (row + gx) * a.c2 + (c - a.c1);
+        cp_async16(smem_addr(dst + v * RSI + c), src, in ? 16 : 0);
+      }
+    };
+    auto load_dy = [&](int y) {
+      bf16* dst = sdy + (y & (YR - 1)) * TV * RSO;
+      const long long row = (long long)a.nx * (y + (long long)a.ny * z);
+      for (int e = tid; e < TV * (CO / 8); e += 256) {
+        const int v = e / (CO / 8), c = (e % (CO / 8)) * 8;
+        const bool in = y < y1 && xs + v < a.nx;
+        cp_async16(smem_addr(dst + v * RSO + c), in ? a.dy + (row + xs + v) * CO + c : a.dy, in ? 16 : 0);
+      }
+    };
+    __syncthreads();  // the previous segment's rows are read
+    load_x(y0 - 1);
+    load_x(y0);
+    load_x(y0 + 1);
+    load_dy(y0);
+    cp_async_commit();
+    load_x(y0 + 2);
+    load_dy(y0 + 1);
+    cp_async_commit();
+    for (int y = y0; y < y1; ++y) {
+      if (y + 2 < y1) {  // the rows of step y + 2
+        load_x(y + 3);
+        load_dy(y + 2);
+      }
+      cp_async_commit();  // (possibly empty)
+      cp_async_wait<2>();
+      __syncthreads();
+      const bf16* dyr = sdy + (y & (YR - 1)) * TV * RSO;
+      if (a.db && dz == 1)
+        for (int v = tid / CO; v < TV; v += 256 / CO) dbs += __bfloat162float(dyr[v * RSO + tid % CO]);
+#pragma unroll
+      for (int k = wk; k < KS; k += WK) {
+        const int kk = k * 16;
+        uint32_t a0, a1, a2, a3;
+        ldsm_x4_t(smem_addr(dyr + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), a0, a1, a2, a3);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          const bf16* xr = sx + ((y + t / 3) & (XR - 1)) * (TV + 2) * RSI + (kk + t % 3) * RSI + nt0 * 8;
+#pragma unroll
+          for (int n = 0; n < NCB; n += 2) {
+            uint32_t b0, b1, b2, b3;
+            if (NCB > 1) {  // two 8-channel columns per load
+              ldsm_x4_t(smem_addr(xr + ((q & 1) * 8 + r) * RSI + n * 8 + (q >> 1) * 8), b0, b1, b2, b3);
+              mma_bf16(acc[t][n], a0, a1, a2, a3, b0, b1);
+              mma_bf16(acc[t][n + 1 < NCB ? n + 1 : n], a0, a1, a2, a3, b2, b3);
+            } else {
+              ldsm_x2_t(smem_addr(xr + (lane & 15) * RSI), b0, b1);
+              mma_bf16(acc[t][n], a0, a1, a2, a3, b0, b1);
+            }
+          }
         }
       }
-      *reinterpret_cast<uint4*>(sx + vi * RSI + c8 * 8) = val;
+      __syncthreads();  // row y - 1 of X and row y of dY are refilled two steps on
     }
-    __syncthreads();
-    if (a.db && tap == 13 && tid < CO)
-      for (int vi = 0; vi < TV; ++vi) dbs += __bfloat162float(sdy[vi * RSO + tid]);
-#pragma unroll
-    for (int j = 0; j < NACC; ++j) {
-      const int tile = TILES >= 8 ? warp + 8 * j : warp % TILES;
-      const int mt = tile / NT, nt = tile % NT;
-      // K-steps of this warp for this tile: all four, or (with fewer tiles than warps) every 8/TILES-th
-      constexpr int KSTEP = TILES >= 8 ? 1 : 8 / TILES;
-      const int k_first = TILES >= 8 ? 0 : warp / TILES;
-#pragma unroll
-      for (int ks = k_first; ks < TV / 16; ks += KSTEP) {
-        const int kk = ks * 16;
-        uint32_t a0, a1, a2, a3, b0, b1;
-        ldsm_x4_t(smem_addr(sdy + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), a0, a1, a2, a3);
-        ldsm_x2_t(smem_addr(sx + (kk + (lane & 15)) * RSI + nt * 8), b0, b1);
-        mma_bf16(acc[j], a0, a1, a2, a3, b0, b1);
-      }
-    }
+    cp_async_wait<0>();
   }
   const int cin = a.c1 + a.c2;
+  float* dw = a.dw + (long long)dz * 9 * CO * cin;
+  const int m = mt * 16 + (lane >> 2), n2 = 2 * (lane & 3);
+  if (WK > 1) {  // the voxel shares add up in shared memory, one after the other
+    float* sum = (float*)wg_smem;
+    for (int w = 0; w < WK; ++w) {
+      __syncthreads();
+      if (wk == w) {
 #pragma unroll
-  for (int j = 0; j < NACC; ++j) {
-    const int tile = TILES >= 8 ? warp + 8 * j : warp % TILES;
-    const int mt = tile / NT, nt = tile % NT;
-    const int m = mt * 16 + (lane >> 2), n = nt * 8 + 2 * (lane & 3);
-    float* w0 = a.dw + ((long long)tap * CO + m) * cin + n;
-    atomicAdd(w0, acc[j][0]);
-    atomicAdd(w0 + 1, acc[j][1]);
-    atomicAdd(w0 + 8LL * cin, acc[j][2]);
-    atomicAdd(w0 + 8LL * cin + 1, acc[j][3]);
+        for (int t = 0; t < 9; ++t)
+#pragma unroll
+          for (int n = 0; n < NCB; ++n) {
+            float* p0 = sum + (t * CO + m) * CI + (nt0 + n) * 8 + n2;
+            float* p1 = p0 + 8 * CI;
+            p0[0] = w ? p0[0] + acc[t][n][0] : acc[t][n][0];
+            p0[1] = w ? p0[1] + acc[t][n][1] : acc[t][n][1];
+            p1[0] = w ? p1[0] + acc[t][n][2] : acc[t][n][2];
+            p1[1] = w ? p1[1] + acc[t][n][3] : acc[t][n][3];
+          }
+      }
+    }
+    __syncthreads();
+    if (((uintptr_t)dw & 15) == 0) {
+      for (int e = tid; e < 9 * CO * CI / 4; e += 256)
+        atomicAdd(reinterpret_cast<float4*>(dw) + e, reinterpret_cast<const float4*>(sum)[e]);
+    } else {
+      for (int e = tid; e < 9 * CO * CI; e += 256) atomicAdd(dw + e, sum[e]);
+    }
+  } else {
+    const bool pairs = ((uintptr_t)dw & 7) == 0;
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+#pragma unroll
+      for (int n = 0; n < NCB; ++n) {
+        float* p0 = dw + (t * CO + m) * CI + (nt0 + n) * 8 + n2;
+        float* p1 = p0 + 8 * CI;
+        if (pairs) {
+          atomicAdd(reinterpret_cast<float2*>(p0), make_float2(acc[t][n][0], acc[t][n][1]));
+          atomicAdd(reinterpret_cast<float2*>(p1), make_float2(acc[t][n][2], acc[t][n][3]));
+        } else {
+          atomicAdd(p0, acc[t][n][0]);
+          atomicAdd(p0 + 1, acc[t][n][1]);
+          atomicAdd(p1, acc[t][n][2]);
+          atomicAdd(p1 + 1, acc[t][n][3]);
+        }
+      }
   }
-  if (a.db && tap == 13 && tid < CO) atomicAdd(&a.db[tid], dbs);
+  if (a.db && dz == 1) {
+#pragma unroll
+    for (int o = CO; o < 32; o *= 2) dbs += __shfl_xor_sync(0xffffffffu, dbs, o);
+    if (lane < CO) atomicAdd(&a.db[tid % CO], dbs);
+  }
 }
 
 // ---- pooling ------------------------------------------------------------------------------------
