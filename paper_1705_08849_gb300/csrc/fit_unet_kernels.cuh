@@ -298,6 +298,14 @@ __device__ inline void tc_tma_load_5d(uint32_t dst, const CUtensorMap* tm, int c
 __device__ inline void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+// the same by one lane of a warp that runs in step (leader != 0 in that lane alone)
+__device__ inline void tc_commit_by(uint32_t bar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+      "r"(leader)
+      : "memory");
+}
 // 16 consecutive FP32 columns of this warp's 32 TMEM lanes
 __device__ inline void tc_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
@@ -317,13 +325,15 @@ __device__ inline void tc_st16_zero(uint32_t taddr) {
       "r"(z)
       : "memory");
 }
-// one MMA of M = 128 into TMEM columns dcol.., N = n (16 .. 256, a multiple of 16), accumulating
-__device__ inline void tc_mma_acc(uint32_t dcol, uint64_t ad, uint64_t bd, int n) {
-  const uint32_t idesc = tc_idesc_bf16(128, 0) | ((uint32_t)(n >> 3) << 17);
+// one MMA of M = 128 into TMEM columns dcol.., accumulating; idesc from tc_idesc_bf16(128, n), n = 16 .. 256 a
+// multiple of 16.  The whole warp calls it with the same values and the leader lane issues it: the operands
+// of tcgen05.mma live in uniform registers, and computed by one lane in a branch of its own every one of them
+// had to be moved there first.
+__device__ inline void tc_mma_acc(uint32_t dcol, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dcol),
-      "l"(ad), "l"(bd), "r"(idesc), "r"(1u)
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %4, 0;\n\tsetp.ne.u32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dcol),
+      "l"(ad), "l"(bd), "r"(idesc), "r"(1u), "r"(leader)
       : "memory");
 }
 
@@ -393,7 +403,7 @@ __global__ void __launch_bounds__(192) conv3_tc_kernel(const __grid_constant__ C
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform, for the MMA warp's operands)
   if (warp >= 2) {  // every accumulator block starts at zero (all MMAs accumulate)
     const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
 #pragma unroll
@@ -430,46 +440,49 @@ __global__ void __launch_bounds__(192) conv3_tc_kernel(const __grid_constant__ C
       for (int d = 1; d <= S && d <= i; ++d) (void)tc_mbar_wait(full((i - d) % S), ((i - d) / S) & 1);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      const uint64_t bdesc = tc_smem_desc(w_s, N3 * 16, 128);
-      for (int i = 0; i < nplanes; ++i) {
-        // plane i feeds outputs j = i - dz for dz in [dz_lo, dz_hi] (those inside the chunk)
-        const int dz_lo = max(0, i - (nout - 1)), dz_hi = min(2, i);
-        bool ok = tc_mbar_wait(full(i % S), (i / S) & 1, stop);
-        if (ok && dz_lo == 0 && i >= R) ok = tc_mbar_wait(acce(i % R), ((i / R) - 1) & 1, stop);  // block of output i free
-        if (!ok) {
-          fail();
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // the dz range in at most two runs of adjacent blocks: the ring wraps after the output whose
-        // block is R-1 (j % R == 0), at most once in three outputs (R >= 4)
-        int brk = -1;
-        for (int dz = dz_lo; dz < dz_hi; ++dz)
-          if ((i - dz) % R == 0) brk = dz;
-        const int a1 = dz_lo, b1 = brk >= 0 ? brk : dz_hi;  // first run
-        const int a2 = b1 + 1;                                // second run: a2 .. dz_hi when brk >= 0
-        const uint64_t adesc = tc_smem_desc(ring + (i % S) * SH::PLANE, SH::GROUP, SH::PX * 16);
+    // ---------------- MMA issuer: the warp in step, lane 0 issues ----------------
+    const uint32_t leader = lane == 0 ? 1u : 0u;
+    const uint64_t bdesc = tc_smem_desc(w_s, N3 * 16, 128);
+    const uint32_t idesc0 = tc_idesc_bf16(128, 0);
+    for (int i = 0; i < nplanes; ++i) {
+      // plane i feeds outputs j = i - dz for dz in [dz_lo, dz_hi] (those inside the chunk)
+      const int dz_lo = max(0, i - (nout - 1)), dz_hi = min(2, i);
+      bool ok = tc_mbar_wait(full(i % S), (i / S) & 1, stop);
+      if (ok && dz_lo == 0 && i >= R) ok = tc_mbar_wait(acce(i % R), ((i / R) - 1) & 1, stop);  // block of output i free
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0) fail();
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // the dz range in at most two runs of adjacent blocks: the ring wraps after the output whose
+      // block is R-1 (j % R == 0), at most once in three outputs (R >= 4)
+      int brk = -1;
+      for (int dz = dz_lo; dz < dz_hi; ++dz)
+        if ((i - dz) % R == 0) brk = dz;
+      const int a1 = dz_lo, b1 = brk >= 0 ? brk : dz_hi;  // first run
+      const int a2 = b1 + 1;                                // second run: a2 .. dz_hi when brk >= 0
+      const uint64_t adesc = tc_smem_desc(ring + (i % S) * SH::PLANE, SH::GROUP, SH::PX * 16);
+      auto run = [&](int lo, int hi) {
+        const uint32_t d = tmem + (uint32_t)(blk(i - lo) * NC);
+        const uint32_t idesc = idesc0 | ((uint32_t)(((hi - lo + 1) * NC) >> 3) << 17);
+        const uint64_t bd = bdesc + (uint64_t)((lo * NC * 16) >> 4);
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
           const int dy = t / 3, dx = t % 3;
 #pragma unroll
-          for (int kk = 0; kk < CIN / 16; ++kk) {
-            const uint64_t ad = adesc + (uint64_t)(((dy * SH::PX + dx) * 16 + kk * 2 * SH::GROUP) >> 4);
-            const uint64_t bt = bdesc + (uint64_t)(((t * CG + 2 * kk) * N3 * 16) >> 4);
-            tc_mma_acc(tmem + (uint32_t)(blk(i - a1) * NC), ad, bt + (uint64_t)((a1 * NC * 16) >> 4), (b1 - a1 + 1) * NC);
-            if (brk >= 0)
-              tc_mma_acc(tmem + (uint32_t)(blk(i - a2) * NC), ad, bt + (uint64_t)((a2 * NC * 16) >> 4),
-                         (dz_hi - a2 + 1) * NC);
-          }
+          for (int kk = 0; kk < CIN / 16; ++kk)
+            tc_mma_acc(d, adesc + (uint64_t)(((dy * SH::PX + dx) * 16 + kk * 2 * SH::GROUP) >> 4),
+                       bd + (uint64_t)(((t * CG + 2 * kk) * N3 * 16) >> 4), idesc, leader);
         }
-        tc_commit(empty(i % S));                   // plane i is no longer read
-        if (dz_hi == 2) tc_commit(accf((i - 2) % R));  // output i-2 has all its contributions
-      }
-      tc_commit(done);  // every MMA this CTA issued has completed once this barrier flips
-      (void)tc_mbar_wait(done, 0);
+      };
+      run(a1, b1);
+      if (brk >= 0) run(a2, dz_hi);
+      tc_commit_by(empty(i % S), leader);                   // plane i is no longer read
+      if (dz_hi == 2) tc_commit_by(accf((i - 2) % R), leader);  // output i-2 has all its contributions
     }
+    tc_commit_by(done, leader);  // every MMA this CTA issued has completed once this barrier flips
+    (void)tc_mbar_wait(done, 0);
+    __syncwarp();
   } else {
     // ---------------- epilogue: warps 2..5 ----------------
     const int q = warp & 3;  // TMEM lanes 32q .. 32q+31 = tile rows 4q .. 4q+3
