@@ -343,6 +343,8 @@ fit_status conv3(const bf16* in1, int c1, const bf16* in2, int c2, const bf16* w
   a.c1 = c1;
   a.c2 = c2;
   a.w = w;
+  a.w32 = nullptr;
+  a.w32_t = 0;
   a.bias = bias;
   a.out1 = out1;
   a.out2 = out2;
@@ -910,33 +912,49 @@ fit_status layer_weights(const float* w, int cin, int cout, bf16** wf, bf16** wt
   FIT_CHECK_CUDA(cudaGetLastError());
   return FIT_OK;
 }
+
+// One conv with a layer's FP32 weights (cin, cout: the layer's), or its data gradient (transposed).  The tcgen05
+// kernels round the weights as they stage them: scratch copies of a call's own cost two stream-ordered
+// allocations, which a synchronising program pays in full every time (180 us), and a 5 us kernel.  The legacy
+// kernels take bf16 copies.
+fit_status conv3_layer(const void* in, const float* w, const float* bias, int relu, void* out, int cin, int cout,
+                       int transposed, int nx, int ny, int nz, cudaStream_t s) {
+  unet::ConvArgs a = {};
+  a.in1 = (const bf16*)in;
+  a.c1 = transposed ? cout : cin;
+  a.w32 = w;
+  a.w32_t = transposed;
+  a.bias = bias;
+  a.out1 = (bf16*)out;
+  a.o1 = a.cout = transposed ? cin : cout;
+  a.nx = nx;
+  a.ny = ny;
+  a.nz = nz;
+  a.relu = relu;
+  bool done = false;
+  fit_status st = conv3_tc(a, a.c1, s, &done);
+  if (done) return st;
+  bf16 *wf = nullptr, *wt = nullptr;
+  UCK(layer_weights(w, cin, cout, &wf, &wt, s));
+  st = conv3(a.in1, a.c1, nullptr, 0, transposed ? wt : wf, bias, a.out1, a.o1, nullptr, 0, nx, ny, nz, relu, s);
+  cudaFreeAsync(wf, s);
+  cudaFreeAsync(wt, s);
+  return st;
+}
 }  // namespace
 
 fit_status fit_unet_conv3(int nx, int ny, int nz, int cin, int cout, const void* in, const float* w, const float* bias,
                           int relu, void* out, void* stream) {
   FIT_REQUIRE(in && w && out && nx >= 1 && ny >= 1 && nz >= 1, "fit_unet_conv3: bad argument");
   FIT_REQUIRE(conv_shape_ok(cin, cout), "fit_unet_conv3: (cin, cout) is not a layer shape of the network");
-  cudaStream_t s = (cudaStream_t)stream;
-  bf16 *wf = nullptr, *wt = nullptr;
-  UCK(layer_weights(w, cin, cout, &wf, &wt, s));
-  fit_status st = conv3((const bf16*)in, cin, nullptr, 0, wf, bias, (bf16*)out, cout, nullptr, 0, nx, ny, nz,
-                        relu ? 1 : 0, s);
-  cudaFreeAsync(wf, s);
-  cudaFreeAsync(wt, s);
-  return st;
+  return conv3_layer(in, w, bias, relu ? 1 : 0, out, cin, cout, 0, nx, ny, nz, (cudaStream_t)stream);
 }
 
 fit_status fit_unet_conv3_dgrad(int nx, int ny, int nz, int cin, int cout, const void* dout, const float* w, void* din,
                                 void* stream) {
   FIT_REQUIRE(dout && w && din && nx >= 1 && ny >= 1 && nz >= 1, "fit_unet_conv3_dgrad: bad argument");
   FIT_REQUIRE(conv_shape_ok(cin, cout), "fit_unet_conv3_dgrad: (cin, cout) is not a layer shape of the network");
-  cudaStream_t s = (cudaStream_t)stream;
-  bf16 *wf = nullptr, *wt = nullptr;
-  UCK(layer_weights(w, cin, cout, &wf, &wt, s));
-  fit_status st = conv3((const bf16*)dout, cout, nullptr, 0, wt, nullptr, (bf16*)din, cin, nullptr, 0, nx, ny, nz, 0, s);
-  cudaFreeAsync(wf, s);
-  cudaFreeAsync(wt, s);
-  return st;
+  return conv3_layer(dout, w, nullptr, 0, din, cin, cout, 1, nx, ny, nz, (cudaStream_t)stream);
 }
 
 fit_status fit_unet_conv3_wgrad(int nx, int ny, int nz, int cin, int cout, const void* in, const void* dout, float* dw,

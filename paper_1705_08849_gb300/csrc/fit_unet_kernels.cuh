@@ -28,6 +28,8 @@ struct ConvArgs {
   const bf16* in2;
   int c1, c2;        // channels of the two inputs (c1 + c2 = CIN)
   const bf16* w;     // [27][cout][CIN]
+  const float* w32;  // or (tcgen05 kernel) the FP32 weights, rounded to bf16 as they are staged:
+  int w32_t;         // 0: [27][cout][CIN]; 1: the forward conv's [27][CIN][cout], taps mirrored (data gradient)
   const float* bias; // [cout] or null
   bf16* out1;
   bf16* out2;
@@ -391,6 +393,18 @@ __global__ void __launch_bounds__(192) conv3_tc_kernel(const __grid_constant__ C
     const int n3 = q % N3, g = (q / N3) % CG, t = q / (N3 * CG);
     const int dz = n3 / NC, n = n3 % NC;
     const bool in = n0 + n < a.cout;
+    if (a.w32) {
+      const int tap = a.w32_t ? 26 - (dz * 9 + t) : dz * 9 + t;
+      const float* src = a.w32_t ? a.w32 + ((long long)tap * CIN + g * 8) * a.cout + n0 + n
+                                 : a.w32 + ((long long)tap * a.cout + n0 + n) * CIN + g * 8;
+      const int step = a.w32_t ? a.cout : 1;
+      __align__(16) __nv_bfloat162 pk[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        pk[e] = in ? __floats2bfloat162_rn(src[2 * e * step], src[(2 * e + 1) * step]) : __floats2bfloat162_rn(0.f, 0.f);
+      *reinterpret_cast<uint4*>(smem + q * 16) = *reinterpret_cast<const uint4*>(pk);
+      continue;
+    }
     const void* src =
         in ? (const void*)(a.w + ((long long)(dz * 9 + t) * a.cout + n0 + n) * CIN + g * 8) : (const void*)a.w;
     cp_async16(w_s + q * 16, src, in ? 16 : 0);
