@@ -290,17 +290,26 @@ static fit_status conv3_tc(const unet::ConvArgs& a, int cin, cudaStream_t s, boo
 }
 
 // Weight gradient of a 3x3x3 conv on the tensor cores: dw (27 x cout x cin) and db accumulate (the caller
-// zeroes them).  Two blocks per SM, a third of them for each z-tap, every one with about three row
+// zeroes them).  One wave of resident blocks, a third of them for each z-tap, every one with about three row
 // segments' worth of y-chunks (at least eight rows each, so that a chunk's two halo rows stay a small part).
 template <int CO, int CI, int TV>
 fit_status wgrad_launch_shape(const unet::WgradArgs& w, cudaStream_t s) {
   auto kern = unet::conv3_wgrad_kernel<CO, CI, TV>;
   constexpr int smem = unet::WgradShape<CO, CI>::smem(TV);
-  int dev = 0, nsm = 0;
-  FIT_CHECK_CUDA(cudaGetDevice(&dev));
-  FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  const int blocks = std::max(1, 2 * nsm / 3);
+  static int slots = 0;  // resident blocks, per instantiation, looked up once
+  if (slots == 0) {
+    int dev = 0, nsm = 0, p = 0;
+    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    FIT_CHECK_CUDA(cudaGetDevice(&dev));
+    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    FIT_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kern, 256, smem));
+    if (p < 1) {
+      fit_set_error("U-Net: weight-gradient tile does not fit on an SM");
+      return FIT_EINVAL;
+    }
+    slots = p * nsm;
+  }
+  const int blocks = std::max(1, slots / 3);
   const long long rows = (long long)((w.nx + TV - 1) / TV) * w.nz;
   const int most = std::max(1, w.ny / 8);
   const int nyc = (int)std::min<long long>(most, std::max(1LL, (3LL * blocks + rows - 1) / rows));
