@@ -59,8 +59,8 @@ def lib():
         L.fit_grid_create.argtypes = [i, i, i, pd, pd, pd, u, ct.POINTER(vp)]
         L.fit_set_materials.argtypes = [vp, pf, pf, pf, pu8]
         L.fit_set_material_matrices.argtypes = [vp, pd, pd, pd, pu8]
-        L.fit_apply.argtypes = [vp, i, pd, vp, vp, i, vp]
-        L.fit_apply_sym.argtypes = [vp, i, pd, vp, vp, i, vp]
+        L.fit_apply.argtypes = [vp, i, vp, vp, vp, i, vp]
+        L.fit_apply_sym.argtypes = [vp, i, vp, vp, vp, i, vp]
         L.fit_apply_sym.restype = ct.c_int
         L.fit_solve.argtypes = [vp, i, pd, vp, vp, d, ct.POINTER(fit_solve_opts), ct.POINTER(fit_solve_report)]
         L.fit_solve_opts_default.argtypes = [ct.POINTER(fit_solve_opts)]
@@ -75,7 +75,7 @@ def lib():
         L.fit_apply_variant_count.restype = ct.c_int
         L.fit_apply_tuned.argtypes = [vp, i, i, ct.POINTER(ct.c_int)]
         L.fit_apply_tuned.restype = ct.c_int
-        L.fit_apply_noalloc.argtypes = [vp, i, pd, vp, vp, i, vp]
+        L.fit_apply_noalloc.argtypes = [vp, i, vp, vp, vp, i, vp]
         L.fit_apply_noalloc.restype = ct.c_int
         L.fit_jacobi.argtypes = [vp, i, pd, vp, vp, i, vp]
         L.fit_jacobi.restype = ct.c_int
@@ -212,40 +212,61 @@ def grid_info(g):
     return dict(nx=out[0], ny=out[1], nz=out[2], ne=out[3], bytes_held=out[4], budget=out[5])
 
 
+_torch_module = None
+
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
 def _check_vec(t, ne, nbatch, prec, name):
-    import torch
+    torch = _torch()
     want = torch.complex64 if prec == FIT_C64 else torch.complex128
     if not (t.is_cuda and t.dtype == want and t.is_contiguous() and t.numel() == ne * nbatch):
         raise ValueError(f"{name} must be a contiguous CUDA {want} tensor of {nbatch} x {ne} values")
 
 
+_Info = ct.c_longlong * 6
+
+
+def _call_apply(call, what, g, ne, omega, x, y, prec, stream):
+    """One apply call.  A pass over a small grid takes the device a few microseconds, so the arguments go
+    through as plain integers and nothing is looked up twice (per call 19.8 us at 16^3 with a dict of the
+    grid's sizes, pointer objects and an import each)."""
+    if type(omega) is not np.ndarray or omega.dtype != np.float64 or omega.ndim != 1 or not omega.flags.c_contiguous:
+        omega = np.ascontiguousarray(np.atleast_1d(np.asarray(omega, dtype=np.float64)))
+    nb = omega.size
+    if ne is None:
+        out = _Info()
+        _check(lib().fit_grid_info(g, out), "fit_grid_info")
+        ne = out[3]
+    _check_vec(x, ne, nb, prec, "x")
+    _check_vec(y, ne, nb, prec, "y")
+    if stream is None:
+        stream = _torch().cuda.current_stream()
+    st = call(g, nb, omega.__array_interface__["data"][0], x.data_ptr(), y.data_ptr(), prec,
+              stream if isinstance(stream, int) else stream.cuda_stream)
+    if st < 0:
+        _check(st, what)
+
+
 def fit_apply(g, omega, x, y, prec=FIT_C64, stream=None):
     """y_b = A(omega_b) x_b for the batch of len(omega) vectors (torch CUDA tensors)."""
-    om, pom = _dptr(np.atleast_1d(np.asarray(omega, dtype=np.float64)), np.float64)
-    ne = grid_info(g)["ne"]
-    _check_vec(x, ne, len(om), prec, "x")
-    _check_vec(y, ne, len(om), prec, "y")
-    _check(lib().fit_apply(g, len(om), pom, ct.c_void_p(x.data_ptr()), ct.c_void_p(y.data_ptr()), prec,
-                           _stream_ptr(stream)), "fit_apply")
+    _call_apply(lib().fit_apply, "fit_apply", g, None, omega, x, y, prec, stream)
 
 
 def fit_apply_sym(g, omega, x, y, prec=FIT_C64, stream=None):
     """y'_b = A_s(omega_b) x'_b, the symmetrised operator M_eps^-1/2 A M_eps^-1/2 of Eq. e2s."""
-    om, pom = _dptr(np.atleast_1d(np.asarray(omega, dtype=np.float64)), np.float64)
-    ne = grid_info(g)["ne"]
-    _check_vec(x, ne, len(om), prec, "x")
-    _check_vec(y, ne, len(om), prec, "y")
-    _check(lib().fit_apply_sym(g, len(om), pom, _ptr(x), _ptr(y), prec, _stream_ptr(stream)), "fit_apply_sym")
+    _call_apply(lib().fit_apply_sym, "fit_apply_sym", g, None, omega, x, y, prec, stream)
 
 
 def fit_apply_noalloc(g, omega, x, y, prec=FIT_C64, stream=None):
     """fit_apply without device allocations (static frequency scratch of 4096 systems)."""
-    om, pom = _dptr(np.atleast_1d(np.asarray(omega, dtype=np.float64)), np.float64)
-    ne = grid_info(g)["ne"]
-    _check_vec(x, ne, len(om), prec, "x")
-    _check_vec(y, ne, len(om), prec, "y")
-    _check(lib().fit_apply_noalloc(g, len(om), pom, ct.c_void_p(x.data_ptr()), ct.c_void_p(y.data_ptr()), prec,
-                                   _stream_ptr(stream)), "fit_apply_noalloc")
+    _call_apply(lib().fit_apply_noalloc, "fit_apply_noalloc", g, None, omega, x, y, prec, stream)
 
 
 def fit_solve_opts_default():
@@ -574,7 +595,7 @@ class Grid:
         return g
 
     def apply(self, omega, x, y, prec=FIT_C64, stream=None):
-        fit_apply(self.h, omega, x, y, prec, stream)
+        _call_apply(lib().fit_apply, "fit_apply", self.h, self.ne, omega, x, y, prec, stream)
 
     def solve(self, omega, rhs, x, tol, **kw):
         return fit_solve(self.h, omega, rhs, x, tol, **kw)
