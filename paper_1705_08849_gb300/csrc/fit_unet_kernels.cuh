@@ -389,25 +389,57 @@ __global__ void __launch_bounds__(192) conv3_tc_kernel(const __grid_constant__ C
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   // weights: line (t, g, dz * NC + n) = W[dz * 9 + t][n0 + n][8g .. 8g+7] (channels beyond cout are zero)
-  for (int q = tid; q < 9 * CG * N3; q += 192) {
-    const int n3 = q % N3, g = (q / N3) % CG, t = q / (N3 * CG);
-    const int dz = n3 / NC, n = n3 % NC;
-    const bool in = n0 + n < a.cout;
-    if (a.w32) {
-      const int tap = a.w32_t ? 26 - (dz * 9 + t) : dz * 9 + t;
-      const float* src = a.w32_t ? a.w32 + ((long long)tap * CIN + g * 8) * a.cout + n0 + n
-                                 : a.w32 + ((long long)tap * a.cout + n0 + n) * CIN + g * 8;
-      const int step = a.w32_t ? a.cout : 1;
-      __align__(16) __nv_bfloat162 pk[4];
+  constexpr int WLINES = 9 * CG * N3;
+  auto wline = [&](int q, int& g, int& tap, int& n) {
+    const int n3 = q % N3, t = q / (N3 * CG);
+    g = (q / N3) % CG;
+    n = n0 + n3 % NC;
+    tap = (n3 / NC) * 9 + t;
+  };
+  if (a.w32) {  // four lines per thread and trip, all loads first: their latency, not their bytes, costs here
+    const bool vec = !a.w32_t && ((uintptr_t)a.w32 & 15) == 0;
+    for (int q0 = tid; q0 < WLINES; q0 += 4 * 192) {
+      float v[4][8];
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        pk[e] = in ? __floats2bfloat162_rn(src[2 * e * step], src[(2 * e + 1) * step]) : __floats2bfloat162_rn(0.f, 0.f);
-      *reinterpret_cast<uint4*>(smem + q * 16) = *reinterpret_cast<const uint4*>(pk);
-      continue;
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + 192 * u;
+        int g, tap, n;
+        wline(q, g, tap, n);
+        const bool in = q < WLINES && n < a.cout;
+        if (vec) {
+          const float4* src = reinterpret_cast<const float4*>(a.w32 + ((long long)tap * a.cout + n) * CIN + g * 8);
+          const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), lo = in ? src[0] : z, hi = in ? src[1] : z;
+          v[u][0] = lo.x, v[u][1] = lo.y, v[u][2] = lo.z, v[u][3] = lo.w;
+          v[u][4] = hi.x, v[u][5] = hi.y, v[u][6] = hi.z, v[u][7] = hi.w;
+        } else {
+          const float* src = a.w32_t ? a.w32 + ((long long)(26 - tap) * CIN + g * 8) * a.cout + n
+                                     : a.w32 + ((long long)tap * a.cout + n) * CIN + g * 8;
+          const int step = a.w32_t ? a.cout : 1;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[u][e] = in ? src[e * step] : 0.f;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = q0 + 192 * u;
+        if (q >= WLINES) break;
+        uint32_t pk[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const __nv_bfloat162 h = __floats2bfloat162_rn(v[u][2 * e], v[u][2 * e + 1]);
+          pk[e] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(smem + q * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
     }
-    const void* src =
-        in ? (const void*)(a.w + ((long long)(dz * 9 + t) * a.cout + n0 + n) * CIN + g * 8) : (const void*)a.w;
-    cp_async16(w_s + q * 16, src, in ? 16 : 0);
+  } else {
+    for (int q = tid; q < WLINES; q += 192) {
+      int g, tap, n;
+      wline(q, g, tap, n);
+      const bool in = n < a.cout;
+      const void* src = in ? (const void*)(a.w + ((long long)tap * a.cout + n) * CIN + g * 8) : (const void*)a.w;
+      cp_async16(w_s + q * 16, src, in ? 16 : 0);
+    }
   }
   cp_async_commit();
   float* bias_s = (float*)(smem + SH::OFF_BIAS);
