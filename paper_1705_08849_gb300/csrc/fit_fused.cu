@@ -529,7 +529,7 @@ __device__ inline void named_barrier(int id, int nthreads) {
 // boundaries at both ends; row (j, p) of the stage is shifted by one value where x's row starts on an odd
 // one.  What the copies leave stale or bring from a neighbouring row lies outside the grid: the mask byte
 // of a cell inside it carries bit 3, so the masking warp zeroes every staged cell without that bit.
-// 149 x 107 x 83: 33.8 us against 76.3 us of the generic kernel.
+// 149 x 107 x 83: 33.7 us against 76.3 us of the generic kernel.
 template <typename V>
 __device__ inline V vadd(V a, V b) {
   if constexpr (sizeof(V) == 8) {
@@ -1195,7 +1195,7 @@ struct Variant {
 //         resident CTAs; with a batch it falls back to tz = 0
 // The CTA-synchronous kernel stays for grids of a few tiles, where a plane's way through the masking warp is
 // the longer one.
-const Variant kVariants64[] = {
+constexpr Variant kVariants64[] = {
     {8, 0, 4, 0, 1},  {8, -1, 4, 0, 1}, {8, 32, 4, 0, 1}, {8, 16, 4, 0, 1},
     // CTA-synchronous
     {4, 0, 3, 0, 0},  {8, 0, 3, 0, 0},  {4, 0, 4, 0, 0},  {8, 0, 4, 0, 0},  {8, 16, 4, 0, 0}, {4, 32, 4, 0, 0},
@@ -1655,6 +1655,22 @@ static fit_status launch_choice(fit_grid* g, int choice, int nbatch, const fit_o
   return launch_fused<double>(g, nbatch, om, x, y, g->nu64, g->ek64, out_scale, s, e, v[choice]);
 }
 
+// The launch shape of complex64 grids with an odd nx, by rule: only the warp-specialised shapes take them, and
+// four-row tiles win throughout (a plane's rows are copied one by one, and three CTAs per SM overlap more of
+// them).  One system or few tiles: the even split, or balanced chunks; a batch with at least two waves of
+// 32-plane tiles: those, whose CTAs march in step over the systems of a column and share its coefficients in L2.
+// Best of all shapes against this rule: 15x17x13 10.8 / 10.8 us, 63x61x59 11.8 / 13.0, 149x107x83 33.7 / 33.7,
+// 255x251x191 235.7 / 241.8, 41x37x29 x 8 21.2 / 21.2, 95x97x93 x 8 134.3 / 134.3.  A search would cost the
+// first apply 34 ms.
+static int odd_choice(const fit_grid* g, int nbatch) {
+  constexpr int kEven = 21, kChunks = 20;
+  static_assert(kVariants64[kEven].ty == 4 && kVariants64[kEven].tz == -1 && kVariants64[kEven].rows == 1 &&
+                    kVariants64[kChunks].ty == 4 && kVariants64[kChunks].tz == 32 && kVariants64[kChunks].rows == 1,
+                "the shapes this rule names");
+  const long long tiles = (long long)((g->nx + TX - 1) / TX) * ((g->ny + 3) / 4) * ((g->nz + 31) / 32) * nbatch;
+  return nbatch > 1 && tiles >= 2 * 3 * 152 ? kChunks : kEven;
+}
+
 // Reads a buffer (grid-stride, 16 bytes a thread per step) so that its lines replace whatever the
 // L2 held; the store is never taken (the buffer holds 0x01 bytes) but keeps the loads alive.
 __global__ void l2_scrub_kernel(const uint4* __restrict__ p, size_t n, uint4* sink) {
@@ -1677,6 +1693,10 @@ fit_status fit_tune_apply(fit_grid* g, int nbatch, const fit_omega& om, const vo
   if (g->tuned.count(key)) return FIT_OK;
   if (!fused_supported(g, prec)) {
     g->tuned[key] = -1;
+    return FIT_OK;
+  }
+  if (prec == FIT_C64 && g->nx % 2 != 0) {  // (no search: see odd_choice)
+    g->tuned[key] = odd_choice(g, nbatch);
     return FIT_OK;
   }
   // opt-in persistence: a cache file named by FIT_TUNE_CACHE supplies the choice for this device, grid,

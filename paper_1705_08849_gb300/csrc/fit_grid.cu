@@ -445,8 +445,12 @@ fit_status fit_apply(fit_grid* g, int nbatch, const double* omega, const void* x
   cudaStream_t s = (cudaStream_t)stream;
   double out_scale = prec == FIT_C64 ? 1.0 / g->coef_scale : 1.0;
   // A small batch's frequencies travel as kernel arguments: a copy of 8 bytes in front of every apply cost the
-  // host more than the launch and stood between the kernels of consecutive applies on the device.
-  if (nbatch <= FIT_OMEGA_ARGS)
+  // host more than the launch and stood between the kernels of consecutive applies on the device.  A captured
+  // apply keeps the copy: its graph reads the caller's array anew at every replay.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (nbatch <= FIT_OMEGA_ARGS && s && s != cudaStreamLegacy && s != cudaStreamPerThread)
+    FIT_CHECK_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (nbatch <= FIT_OMEGA_ARGS && s != cudaStreamPerThread && cap == cudaStreamCaptureStatusNone)
     return fit_launch_apply(g, nbatch, fit_omega::of_host(omega), x, y, prec, out_scale, s);
   fit_status st = fit_stage_omega(g, nbatch, omega, s);
   if (st != FIT_OK) return st;
