@@ -249,7 +249,8 @@ int fit_apply_variant_count(fit_prec prec);
  *               split evenly over the resident CTAs) of that kernel
  *   out7[4] = shared-memory ring stages (0 for the generic kernel)
  *   out7[5] = 0 generic or CTA-synchronous fused kernel, 1 warp-specialised fused kernel
- *             (a copy-issuing warp and a masking warp feed the ring, one consumer warp per row)
+ *             (a copy-issuing warp and a masking warp feed the ring; a consumer warp owns one tile row, in
+ *             complex128 two)
  *   out7[6] = L2 prefetch distance: planes of the tile requested into L2 this far ahead of
  *             their copy into shared memory (0: none).
  * The autotuner runs on the first fit_apply / fit_solve with a new (prec, nbatch); it times every
@@ -317,8 +318,9 @@ fit_status fit_unet_unpack(const fit_grid* g, const float* y6, double scale, voi
 /* Single layers of the network: the kernels fit_unet_forward and fit_unet_backward run, one call per
  * layer, for per-layer checks and tools.  All tensors are DEVICE pointers in NDHWC layout (voxel
  * x + nx*(y + ny*z), channels innermost); activations are bf16, weights, biases and weight gradients
- * FP32.  Asynchronous on stream.  The convolution calls convert the FP32 weights to the layer's bf16
- * copies in stream-ordered scratch (cudaMallocAsync / cudaFreeAsync) exactly as the network does.
+ * FP32.  Asynchronous on stream.  The convolution kernels round the FP32 weights to bf16 as they stage
+ * them, to the values of the network's bf16 copies (the legacy kernels of FIT_CONV=mma take such copies, in
+ * stream-ordered scratch).
  * FIT_EINVAL for a (cin, cout) that is not a layer shape of the network. */
 /* fit_unet_conv3 -- 3x3x3 convolution, stride 1, zero padding 1, on the tensor cores (bf16 operands, FP32
  * accumulation, bf16 result):  out[v][co] = act(bias[co] + sum_{tap, ci} in[v + off(tap)][ci] W[tap][co][ci])
