@@ -702,25 +702,53 @@ __global__ void __launch_bounds__(256) conv3_wgrad_kernel(WgradArgs a, int ylen,
       const bf16* dyr = sdy + (y & (YR - 1)) * TV * RSO;
       if (a.db && dz == 1)
         for (int v = tid / CO; v < TV; v += 256 / CO) dbs += __bfloat162float(dyr[v * RSO + tid % CO]);
+      auto load_a = [&](int kk, uint32_t (&f)[4]) {
+        ldsm_x4_t(smem_addr(dyr + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), f[0], f[1], f[2], f[3]);
+      };
+      auto xrow = [&](int t, int kk) {
+        return sx + ((y + t / 3) & (XR - 1)) * (TV + 2) * RSI + (kk + t % 3) * RSI + nt0 * 8;
+      };
+      if constexpr (NCB > 1) {  // two 8-channel columns per fragment load
 #pragma unroll
-      for (int k = wk; k < KS; k += WK) {
-        const int kk = k * 16;
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4_t(smem_addr(dyr + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), a0, a1, a2, a3);
+        for (int k = wk; k < KS; k += WK) {
+          uint32_t fa[4];
+          load_a(k * 16, fa);
 #pragma unroll
-        for (int t = 0; t < 9; ++t) {
-          const bf16* xr = sx + ((y + t / 3) & (XR - 1)) * (TV + 2) * RSI + (kk + t % 3) * RSI + nt0 * 8;
+          for (int t = 0; t < 9; ++t) {
+            const bf16* xr = xrow(t, k * 16);
 #pragma unroll
-          for (int n = 0; n < NCB; n += 2) {
-            uint32_t b0, b1, b2, b3;
-            if (NCB > 1) {  // two 8-channel columns per load
+            for (int n = 0; n < NCB; n += 2) {
+              uint32_t b0, b1, b2, b3;
               ldsm_x4_t(smem_addr(xr + ((q & 1) * 8 + r) * RSI + n * 8 + (q >> 1) * 8), b0, b1, b2, b3);
-              mma_bf16(acc[t][n], a0, a1, a2, a3, b0, b1);
-              mma_bf16(acc[t][n + 1 < NCB ? n + 1 : n], a0, a1, a2, a3, b2, b3);
-            } else {
-              ldsm_x2_t(smem_addr(xr + (lane & 15) * RSI), b0, b1);
-              mma_bf16(acc[t][n], a0, a1, a2, a3, b0, b1);
+              mma_bf16(acc[t][n], fa[0], fa[1], fa[2], fa[3], b0, b1);
+              mma_bf16(acc[t][n + 1], fa[0], fa[1], fa[2], fa[3], b2, b3);
             }
+          }
+        }
+      } else if constexpr (KS >= 2 * WK) {  // one column: two of the warp's 16-voxel steps per load
+#pragma unroll
+        for (int k = wk; k < KS; k += 2 * WK) {
+          uint32_t fa[4], fb[4];
+          load_a(k * 16, fa);
+          load_a((k + WK) * 16, fb);
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            uint32_t b0, b1, b2, b3;
+            ldsm_x4_t(smem_addr(xrow(t, (k + (q >> 1) * WK) * 16) + ((q & 1) * 8 + r) * RSI), b0, b1, b2, b3);
+            mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
+            mma_bf16(acc[t][0], fb[0], fb[1], fb[2], fb[3], b2, b3);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int k = wk; k < KS; k += WK) {
+          uint32_t fa[4];
+          load_a(k * 16, fa);
+#pragma unroll
+          for (int t = 0; t < 9; ++t) {
+            uint32_t b0, b1;
+            ldsm_x2_t(smem_addr(xrow(t, k * 16) + (lane & 15) * RSI), b0, b1);
+            mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
           }
         }
       }
