@@ -616,8 +616,8 @@ __device__ inline void ldsm_x2_t(uint32_t addr, uint32_t& r0, uint32_t& r1) {
 // taps' accumulators stay in registers over all of the block's segments: the eight warps are WT groups of
 // (16 output channel) x (8 NCB input channel) columns times WK shares of the segment's voxels.  Rows arrive
 // by cp.async two steps ahead (zero fill outside the grid).  What bounds it: the MMAs and their ldmatrix
-// traffic (one B fragment per MMA for NCB = 1); the final adds are vector reductions to L2, one set per
-// block.  32 -> 16 at 64^3: 221 us with a block per (1024 voxels, tap), each re-reading X and dY and
+// traffic (one four-matrix load per two MMAs); the final adds are vector reductions to L2, one set per
+// block.  32 -> 16 at 64^3: 43 us; 221 us with a block per (1024 voxels, tap), each re-reading X and dY and
 // dividing out every voxel's coordinates.
 template <int CO, int CI>
 struct WgradShape {
