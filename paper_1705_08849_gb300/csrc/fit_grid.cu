@@ -215,17 +215,22 @@ fit_status fit_take_device_error(fit_grid* g) {
   return FIT_ETIMEOUT;
 }
 
-// the batch's frequencies into the handle's device buffer (grown on demand, counted in the budget)
+// room for the batch's frequencies in the handle's device buffer (grown on demand, counted in the budget)
+static fit_status reserve_omega(fit_grid* g, int nbatch) {
+  if (nbatch <= g->omega_cap) return FIT_OK;
+  if (g->omega_dev) fit_dev_free(g, g->omega_dev, g->omega_cap * sizeof(double));
+  g->omega_dev = nullptr;
+  g->omega_cap = 0;
+  const int cap = std::max(nbatch, 64);
+  fit_status st = fit_dev_alloc(g, (void**)&g->omega_dev, cap * sizeof(double));
+  if (st != FIT_OK) return st;
+  g->omega_cap = cap;
+  return FIT_OK;
+}
+
 fit_status fit_stage_omega(fit_grid* g, int nbatch, const double* omega, cudaStream_t s) {
-  if (nbatch > g->omega_cap) {
-    if (g->omega_dev) fit_dev_free(g, g->omega_dev, g->omega_cap * sizeof(double));
-    g->omega_dev = nullptr;
-    g->omega_cap = 0;
-    int cap = std::max(nbatch, 64);
-    fit_status st = fit_dev_alloc(g, (void**)&g->omega_dev, cap * sizeof(double));
-    if (st != FIT_OK) return st;
-    g->omega_cap = cap;
-  }
+  fit_status st = reserve_omega(g, nbatch);
+  if (st != FIT_OK) return st;
   FIT_CHECK_CUDA(cudaMemcpyAsync(g->omega_dev, omega, nbatch * sizeof(double), cudaMemcpyHostToDevice, s));
   return FIT_OK;
 }
@@ -450,8 +455,12 @@ fit_status fit_apply(fit_grid* g, int nbatch, const double* omega, const void* x
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (nbatch <= FIT_OMEGA_ARGS && s && s != cudaStreamLegacy && s != cudaStreamPerThread)
     FIT_CHECK_CUDA(cudaStreamIsCapturing(s, &cap));
-  if (nbatch <= FIT_OMEGA_ARGS && s != cudaStreamPerThread && cap == cudaStreamCaptureStatusNone)
+  if (nbatch <= FIT_OMEGA_ARGS && s != cudaStreamPerThread && cap == cudaStreamCaptureStatusNone) {
+    // (the buffer all the same, once per handle: a later captured apply must not allocate)
+    fit_status st = reserve_omega(g, nbatch);
+    if (st != FIT_OK) return st;
     return fit_launch_apply(g, nbatch, fit_omega::of_host(omega), x, y, prec, out_scale, s);
+  }
   fit_status st = fit_stage_omega(g, nbatch, omega, s);
   if (st != FIT_OK) return st;
   return fit_launch_apply(g, nbatch, g->omega_dev, x, y, prec, out_scale, s);
