@@ -95,9 +95,23 @@ fit_status fit_set_material_matrices(fit_grid* g, const double* m_eps, const dou
  *   x, y     DEVICE arrays of nbatch * n_e complex values of precision prec; must not overlap
  *   prec     FIT_C64 (float2 vectors, FP32 arithmetic) or FIT_C128 (double2, FP64 arithmetic)
  *   stream   cudaStream_t (as void*) on which the kernel is enqueued; asynchronous
+ * Captured into a CUDA graph, the call records a copy node that reads the omega array anew at every replay:
+ * the array must stay valid until the last graph holding the node is destroyed, and writing to it between
+ * replays changes the frequencies.  (Outside a capture the array is no longer needed on return.)  The same
+ * goes for fit_apply_sym, fit_apply_noalloc and fit_jacobi.
  * FIT_EINVAL on bad arguments. */
 fit_status fit_apply(fit_grid* g, int nbatch, const double* omega, const void* x, void* y,
                      fit_prec prec, void* stream);
+
+/* fit_capture_hold, fit_capture_released -- for bindings, whose frequency arrays may be temporaries: learn how
+ * long a captured call's host array is needed.  fit_capture_hold ties token to the graph that stream (a
+ * cudaStream_t as void*) is being captured into and to every graph cloned or instantiated from it, and
+ * returns 1; it returns 0 and does nothing if the stream is not being captured, a negative fit_status on failure.
+ * fit_capture_released writes up to cap tokens whose graphs have all been destroyed, each token once, and
+ * returns their number.  Both thread-safe; the runtime reports a destroyed graph from a thread of its own, so a
+ * token may come a little later. */
+int fit_capture_hold(void* stream, long long token);
+int fit_capture_released(long long* tokens, int cap);
 
 /* fit_apply_sym -- y'_b = A_s(omega_b) x'_b with the symmetrised operator of Eq. e2s (Sec. II,
  * change of variable e' = M_eps^{1/2} e; Eq. e2tt writes the same operator as cal_A^T cal_A - w^2 I

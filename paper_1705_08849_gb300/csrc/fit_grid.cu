@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -235,7 +236,48 @@ fit_status fit_stage_omega(fit_grid* g, int nbatch, const double* omega, cudaStr
   return FIT_OK;
 }
 
+// Tokens of captured calls whose graphs are gone (fit_capture_hold).  Never destroyed: the runtime's thread may
+// report a graph while the process exits.
+struct ReleasedTokens {
+  std::mutex mu;
+  std::vector<long long> list;
+};
+static ReleasedTokens& released_tokens() {
+  static ReleasedTokens* r = new ReleasedTokens();
+  return *r;
+}
+static void CUDART_CB release_token(void* token) {
+  ReleasedTokens& r = released_tokens();
+  std::lock_guard<std::mutex> lock(r.mu);
+  r.list.push_back((long long)(intptr_t)token);
+}
+
 extern "C" {
+
+int fit_capture_hold(void* stream, long long token) {
+  cudaStream_t s = (cudaStream_t)stream;
+  if (!s || s == cudaStreamLegacy) return 0;  // (the legacy stream cannot be captured)
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  FIT_CHECK_CUDA(cudaStreamGetCaptureInfo(s, &status, nullptr, &graph, nullptr, nullptr, nullptr));
+  if (status != cudaStreamCaptureStatusActive) return 0;
+  cudaUserObject_t obj;
+  FIT_CHECK_CUDA(cudaUserObjectCreate(&obj, (void*)(intptr_t)token, release_token, 1, cudaUserObjectNoDestructorSync));
+  const cudaError_t e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+  if (e != cudaSuccess) (void)cudaUserObjectRelease(obj, 1);
+  FIT_CHECK_CUDA(e);
+  return 1;
+}
+
+int fit_capture_released(long long* tokens, int cap) {
+  if (!tokens || cap < 1) return 0;
+  ReleasedTokens& r = released_tokens();
+  std::lock_guard<std::mutex> lock(r.mu);
+  const int n = (int)std::min<size_t>(r.list.size(), (size_t)cap);
+  std::copy(r.list.end() - n, r.list.end(), tokens);
+  r.list.resize(r.list.size() - n);
+  return n;
+}
 
 const char* fit_status_str(fit_status s) {
   switch (s) {

@@ -9,7 +9,9 @@ raises: there is no fallback path.
 from __future__ import annotations
 
 import ctypes as ct
+import itertools
 import os
+import threading
 
 import numpy as np
 
@@ -77,6 +79,10 @@ def lib():
         L.fit_apply_tuned.restype = ct.c_int
         L.fit_apply_noalloc.argtypes = [vp, i, vp, vp, vp, i, vp]
         L.fit_apply_noalloc.restype = ct.c_int
+        L.fit_capture_hold.argtypes = [vp, ct.c_longlong]
+        L.fit_capture_hold.restype = ct.c_int
+        L.fit_capture_released.argtypes = [ct.POINTER(ct.c_longlong), i]
+        L.fit_capture_released.restype = ct.c_int
         L.fit_jacobi.argtypes = [vp, i, pd, vp, vp, i, vp]
         L.fit_jacobi.restype = ct.c_int
         L.fit_coef_scale.argtypes = [vp, ct.POINTER(ct.c_double)]
@@ -232,6 +238,29 @@ def _check_vec(t, ne, nbatch, prec, name):
 
 _Info = ct.c_longlong * 6
 
+# Frequency arrays that a CUDA graph copies from at every replay (token -> array): a captured call records
+# the array's address, so the array stays here until the last graph that holds the copy is destroyed.
+_held = {}
+_held_lock = threading.Lock()
+_held_tokens = itertools.count(1)
+_Tokens = ct.c_longlong * 64
+
+
+def _hold_for_graph(omega, stream):
+    """Keeps omega alive with the graph that `stream` is captured into; nothing to do if it is not."""
+    with _held_lock:
+        token = next(_held_tokens)
+        if _check(lib().fit_capture_hold(stream, token), "fit_capture_hold") == 0:
+            return
+        _held[token] = omega
+        gone = _Tokens()
+        while True:
+            n = lib().fit_capture_released(gone, len(gone))
+            for t in gone[:n]:
+                _held.pop(t, None)
+            if n < len(gone):
+                return
+
 
 def _call_apply(call, what, g, ne, omega, x, y, prec, stream):
     """One apply call.  A pass over a small grid takes the device a few microseconds, so the arguments go
@@ -246,16 +275,22 @@ def _call_apply(call, what, g, ne, omega, x, y, prec, stream):
         ne = out[3]
     _check_vec(x, ne, nb, prec, "x")
     _check_vec(y, ne, nb, prec, "y")
-    if stream is None:
+    own = stream is None
+    if own:
         stream = _torch().cuda.current_stream()
-    st = call(g, nb, omega.__array_interface__["data"][0], x.data_ptr(), y.data_ptr(), prec,
-              stream if isinstance(stream, int) else stream.cuda_stream)
+    if not isinstance(stream, int):
+        stream = stream.cuda_stream
+    if not own or _torch().cuda.is_current_stream_capturing():
+        _hold_for_graph(omega, stream)
+    st = call(g, nb, omega.__array_interface__["data"][0], x.data_ptr(), y.data_ptr(), prec, stream)
     if st < 0:
         _check(st, what)
 
 
 def fit_apply(g, omega, x, y, prec=FIT_C64, stream=None):
-    """y_b = A(omega_b) x_b for the batch of len(omega) vectors (torch CUDA tensors)."""
+    """y_b = A(omega_b) x_b for the batch of len(omega) vectors (torch CUDA tensors).  Captured into a CUDA
+    graph, every replay reads the frequencies anew from the array passed here (from a copy of the values if omega
+    is not a contiguous float64 array), which is kept alive with the graph."""
     _call_apply(lib().fit_apply, "fit_apply", g, None, omega, x, y, prec, stream)
 
 
@@ -331,7 +366,9 @@ def fit_jacobi(g, omega, x, y, prec=FIT_C128, stream=None):
     ne = grid_info(g)["ne"]
     _check_vec(x, ne, len(om), prec, "x")
     _check_vec(y, ne, len(om), prec, "y")
-    _check(lib().fit_jacobi(g, len(om), pom, _ptr(x), _ptr(y), prec, _stream_ptr(stream)), "fit_jacobi")
+    s = _stream_ptr(stream)
+    _hold_for_graph(om, s)
+    _check(lib().fit_jacobi(g, len(om), pom, _ptr(x), _ptr(y), prec, s), "fit_jacobi")
 
 
 def fit_coef_scale(g):
