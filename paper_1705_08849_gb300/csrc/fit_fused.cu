@@ -37,12 +37,11 @@
 #include <string.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
 #include <type_traits>
 #include <vector>
 
 #include "fit_internal.cuh"
+#include "fit_residency.cuh"
 
 namespace {
 
@@ -1214,31 +1213,6 @@ int fused_smem_limit() {
   return v;
 }
 
-// CTAs of one kernel (with its shared memory opted in) resident on the current device at once.  The
-// answers do not change, so they are kept per kernel and device (the two runtime queries cost more than
-// the launch of a small grid).
-template <typename K>
-cudaError_t resident_ctas(K kern, int threads, int smem, long long* slots) {
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, long long> known;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const std::pair<const void*, int> key((const void*)kern, dev);
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = known.find(key);
-  if (it == known.end()) {
-    int per_sm = 0, nsm = 0;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-    if (e != cudaSuccess) return e;
-    it = known.emplace(key, (long long)per_sm * nsm).first;
-  }
-  *slots = it->second;
-  return cudaSuccess;
-}
-
 // launch configuration of a kernel that begins with programmatic_start
 cudaLaunchConfig_t programmatic_config(int grid, dim3 block, int smem, cudaStream_t s, cudaLaunchAttribute* at) {
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1337,8 +1311,9 @@ fit_status launch_variant(fit_grid* g, int nbatch, const fit_omega& om, const vo
   const bool ku = e.mode == FIT_EPI_DOT_U || e.mode == FIT_EPI_RESID;
   int smem = ku ? Layout<T, TY, true>::smem(S) : Layout<T, TY, false>::smem(S);
   auto run = [&](auto kern) -> fit_status {
-    long long slots = 0;
-    FIT_CHECK_CUDA(resident_ctas(kern, (int)(block.x * block.y), smem, &slots));
+    FitResidency res;
+    FIT_CHECK_CUDA(fit_residency((const void*)kern, (int)(block.x * block.y), smem, &res));
+    const long long slots = res.ctas();
     if (slots < 1) {  // shared memory or registers do not allow one resident CTA of this shape
       fit_set_error("fused apply: launch shape does not fit on an SM");
       return FIT_EINVAL;
@@ -1441,8 +1416,9 @@ fit_status launch_rows(fit_grid* g, int nbatch, const fit_omega& om, const void*
   constexpr int smem = L::smem();
   const dim3 block(TX, NCW + 2, 1);
   auto run = [&](auto kern) -> fit_status {
-    long long slots = 0;
-    FIT_CHECK_CUDA(resident_ctas(kern, (int)(block.x * block.y), smem, &slots));
+    FitResidency res;
+    FIT_CHECK_CUDA(fit_residency((const void*)kern, (int)(block.x * block.y), smem, &res));
+    const long long slots = res.ctas();
     if (slots < 1) {
       fit_set_error("fused apply: launch shape does not fit on an SM");
       return FIT_EINVAL;

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "fit_internal.cuh"
+#include "fit_residency.cuh"
 #include "fit_unet_kernels.cuh"
 
 namespace {
@@ -139,23 +140,15 @@ template <int CIN, int NC, int TY>
 fit_status launch_conv3(const unet::ConvArgs& a, cudaStream_t s) {
   auto kern = unet::conv3_kernel<CIN, NC, TY>;
   const int smem = unet::Conv3Shape<CIN, NC, TY>::smem();
-  static int per_sm = 0, nsm = 0;  // per instantiation, looked up once
-  if (per_sm == 0) {
-    int dev = 0;
-    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FIT_CHECK_CUDA(cudaGetDevice(&dev));
-    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    int p = 0;
-    FIT_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kern, 256, smem));
-    if (p < 1) {
-      fit_set_error("U-Net: conv tile does not fit on an SM");
-      return FIT_EINVAL;
-    }
-    per_sm = p;
+  FitResidency res;
+  FIT_CHECK_CUDA(fit_residency((const void*)kern, 256, smem, &res));
+  if (res.per_sm < 1) {
+    fit_set_error("U-Net: conv tile does not fit on an SM");
+    return FIT_EINVAL;
   }
   const int gx = (a.nx + unet::CX - 1) / unet::CX, gy = (a.ny + TY - 1) / TY, nblk = (a.cout + NC - 1) / NC;
   const long long cols = (long long)gx * gy * nblk;
-  const long long per_col = std::max(1LL, (long long)per_sm * nsm / cols);
+  const long long per_col = std::max(1LL, res.ctas() / cols);
   const int tz = (int)std::max(2LL, ((long long)a.nz + per_col - 1) / per_col);
   const int nzc = (a.nz + tz - 1) / tz;
   dim3 grid(gx, gy, (unsigned)(nzc * nblk));
@@ -173,15 +166,14 @@ fit_status tconv_fwd_tc(const bf16* in, const float* w, const float* b, bf16* ou
   using SH = unet::TconvTc<CIN, COUT>;
   auto kern = unet::tconv_tc_kernel<CIN, COUT>;
   constexpr int smem = SH::smem();
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0;
-    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FIT_CHECK_CUDA(cudaGetDevice(&dev));
-    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  }
+  FitResidency res;
+  const auto by_tmem = [](int* per_sm) {
+    *per_sm = SH::PER_SM;
+    return cudaSuccess;
+  };
+  FIT_CHECK_CUDA(fit_residency((const void*)kern, smem, by_tmem, &res));
   const long long ntiles = ((long long)mx * my * mz + 127) / 128;
-  const int grid = (int)std::min<long long>(ntiles, (long long)nsm * SH::PER_SM);
+  const int grid = (int)std::min<long long>(ntiles, res.ctas());
   kern<<<grid, 128, smem, s>>>(in, w, b, out, mx, my, mz);
   FIT_CHECK_CUDA(cudaGetLastError());
   return FIT_OK;
@@ -194,11 +186,8 @@ fit_status tconv_fwd(const bf16* in, const float* w, const float* b, bf16* out, 
   if (conv_use_tc()) return tconv_fwd_tc<CIN, COUT>(in, w, b, out, mx, my, mz, s);
   auto kern = unet::tconv_fwd_kernel<CIN, COUT>;
   constexpr int smem = unet::tconv_smem<CIN, COUT>();
-  static bool attr = false;
-  if (!attr) {
-    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    attr = true;
-  }
+  FitResidency res;  // (for the opt-in: the grid has a thread per output voxel)
+  FIT_CHECK_CUDA(fit_residency((const void*)kern, 256, smem, &res));
   const long long n = 8LL * mx * my * mz;
   kern<<<(unsigned)((n + 255) / 256), 256, smem, s>>>(in, w, b, out, mx, my, mz);
   FIT_CHECK_CUDA(cudaGetLastError());
@@ -226,23 +215,23 @@ fit_status launch_conv3_tc(const unet::ConvArgs& a, cudaStream_t s) {
   // Resident CTAs per SM, from the SM's shared memory (each CTA also reserves 1 KB), its 512 TMEM columns,
   // its 64 K registers and its 2048 threads.  (The runtime's occupancy query answers 1 for this kernel, which left a
   // 128-column grid with one CTA, and one MMA-issuing thread, per SM.)
-  static int per_sm = 0, nsm = 0;
-  if (per_sm == 0) {
+  const auto count = [&](int* per_sm) -> cudaError_t {
     int dev = 0, smem_sm = 0;
-    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FIT_CHECK_CUDA(cudaGetDevice(&dev));
-    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
     cudaFuncAttributes fa;
-    FIT_CHECK_CUDA(cudaFuncGetAttributes(&fa, kern));
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, (const void*)kern);
+    if (e != cudaSuccess) return e;
     const int by_smem = smem_sm / (smem + 1024), by_tmem = 512 / unet::UmmaShape<CIN, NC, S>::TMEM_COLS;
     const int by_regs = 65536 / (192 * ((fa.numRegs + 7) / 8 * 8));
-    const int p = std::min(std::min(by_smem, by_tmem), std::min(by_regs, 2048 / 192));
-    if (p < 1) {
-      fit_set_error("U-Net: tcgen05 conv tile does not fit on an SM");
-      return FIT_EINVAL;
-    }
-    per_sm = p;
+    *per_sm = std::min(std::min(by_smem, by_tmem), std::min(by_regs, 2048 / 192));
+    return cudaSuccess;
+  };
+  FitResidency res;
+  FIT_CHECK_CUDA(fit_residency((const void*)kern, smem, count, &res));
+  if (res.per_sm < 1) {
+    fit_set_error("U-Net: tcgen05 conv tile does not fit on an SM");
+    return FIT_EINVAL;
   }
   CUtensorMap m1, m2;
   if (!conv_tmap(&m1, a.in1, a.c1, a.nx, a.ny, a.nz) || (a.c2 > 0 && !conv_tmap(&m2, a.in2, a.c2, a.nx, a.ny, a.nz))) {
@@ -252,7 +241,7 @@ fit_status launch_conv3_tc(const unet::ConvArgs& a, cudaStream_t s) {
   if (a.c2 == 0) m2 = m1;
   const int gx = (a.nx + TX - 1) / TX, gy = (a.ny + TY - 1) / TY, nblk = (a.cout + NC - 1) / NC;
   const long long cols = (long long)gx * gy * nblk;
-  const long long per_col = std::max(1LL, (long long)per_sm * nsm / cols);
+  const long long per_col = std::max(1LL, res.ctas() / cols);
   const int tz = (int)std::max(2LL, ((long long)a.nz + per_col - 1) / per_col);
   const int nzc = (a.nz + tz - 1) / tz;
   dim3 grid(gx, gy, (unsigned)(nzc * nblk));
@@ -296,20 +285,13 @@ template <int CO, int CI, int TV>
 fit_status wgrad_launch_shape(const unet::WgradArgs& w, cudaStream_t s) {
   auto kern = unet::conv3_wgrad_kernel<CO, CI, TV>;
   constexpr int smem = unet::WgradShape<CO, CI>::smem(TV);
-  static int slots = 0;  // resident blocks, per instantiation, looked up once
-  if (slots == 0) {
-    int dev = 0, nsm = 0, p = 0;
-    FIT_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    FIT_CHECK_CUDA(cudaGetDevice(&dev));
-    FIT_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    FIT_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, kern, 256, smem));
-    if (p < 1) {
-      fit_set_error("U-Net: weight-gradient tile does not fit on an SM");
-      return FIT_EINVAL;
-    }
-    slots = p * nsm;
+  FitResidency res;
+  FIT_CHECK_CUDA(fit_residency((const void*)kern, 256, smem, &res));
+  if (res.per_sm < 1) {
+    fit_set_error("U-Net: weight-gradient tile does not fit on an SM");
+    return FIT_EINVAL;
   }
-  const int blocks = std::max(1, slots / 3);
+  const int blocks = (int)std::max(1LL, res.ctas() / 3);
   const long long rows = (long long)((w.nx + TV - 1) / TV) * w.nz;
   const int most = std::max(1, w.ny / 8);
   const int nyc = (int)std::min<long long>(most, std::max(1LL, (3LL * blocks + rows - 1) / rows));
