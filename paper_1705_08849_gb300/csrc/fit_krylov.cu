@@ -461,6 +461,26 @@ constexpr int VU = 2;
 #define VEC_EACH(p) \
   _Pragma("unroll") for (int u = 0; u < VU; ++u) if (const long long e = e0 + u * es; e < (p).ne)
 
+// A thread's share of a dot product or norm.  How many terms that is depends on the grid of the pass, and so
+// on how many systems share the call: FP32 terms are added as a pair with the exact rounding error of every addition
+// (Knuth's two-sum), whose total carries one rounding whatever its length.  (Six FP32 additions a term, of which an
+// SM does 128 per clock while HBM brings it less than one element: COCG at 128^3 127.1 -> 127.8 us per iteration, 8
+// BiCGStab systems of 40x36x28 63.2 -> 64.0.)  FP64 terms are added plainly.
+template <typename T>
+struct RunSum {
+  T hi = T(0), lo = T(0);
+  __device__ void add(T v) {
+    if constexpr (sizeof(T) == 4) {
+      const T s = hi + v, w = s - hi;
+      lo += (hi - (s - w)) + (v - w);
+      hi = s;
+    } else {
+      hi += v;
+    }
+  }
+  __device__ T value() const { return isfinite(hi) ? hi + lo : hi; }
+};
+
 __global__ void __launch_bounds__(256) k_outer_init(const double2* __restrict__ rhs, double2* __restrict__ x,
                                                     double2* __restrict__ r, double* part, P p) {
   const int b = blockIdx.y;
@@ -619,7 +639,7 @@ __global__ void __launch_bounds__(256) k_bicg_xr(typename cplx<T>::t* d, const t
   if (sys[b].inner_status != SYS_RUN) return;
   const long long off = (long long)b * p.ne;
   const T ar = (T)sys[b].alpha.x, ai = (T)sys[b].alpha.y, orr = (T)sys[b].omega.x, oi = (T)sys[b].omega.y;
-  T acc[3] = {T(0), T(0), T(0)};
+  RunSum<T> sum[3];
   VEC_TRIP(p) {
     V s[VU], pp[VU], tt[VU], dd[VU], rh[VU], sx[VU];
     VEC_EACH(p) {
@@ -638,11 +658,12 @@ __global__ void __launch_bounds__(256) k_bicg_xr(typename cplx<T>::t* d, const t
       rn.y = s[u].y - (orr * tt[u].y + oi * tt[u].x);
       d[off + e] = dd[u];
       r[off + e] = rn;
-      acc[0] += rh[u].x * rn.x + rh[u].y * rn.y;
-      acc[1] += rh[u].x * rn.y - rh[u].y * rn.x;
-      acc[2] += rn.x * rn.x + rn.y * rn.y;
+      sum[0].add(rh[u].x * rn.x + rh[u].y * rn.y);
+      sum[1].add(rh[u].x * rn.y - rh[u].y * rn.x);
+      sum[2].add(rn.x * rn.x + rn.y * rn.y);
     }
   }
+  T acc[3] = {sum[0].value(), sum[1].value(), sum[2].value()};
   fit_block_sum<T, 3>(acc, part + PSLOT(p, b));
   last_block_fin<3>(part, cnt, sys, p, b, OpRho{});
 }
@@ -799,7 +820,7 @@ __global__ void __launch_bounds__(256) k_cocg_r(typename cplx<T>::t* __restrict_
   if (sys[b].inner_status != SYS_RUN) return;
   const long long off = (long long)b * p.ne;
   const T ar = (T)sys[b].alpha.x, ai = (T)sys[b].alpha.y;
-  T acc[3] = {T(0), T(0), T(0)};
+  RunSum<T> sum[3];
   VEC_TRIP(p) {
     V qq[VU], rr[VU], dd[VU];
     VEC_EACH(p) {
@@ -812,11 +833,12 @@ __global__ void __launch_bounds__(256) k_cocg_r(typename cplx<T>::t* __restrict_
       rr[u].y -= ar * qq[u].y + ai * qq[u].x;
       r[off + e] = rr[u];
       const V z = dinv ? cmulv(dd[u], rr[u]) : rr[u];
-      acc[0] += rr[u].x * z.x - rr[u].y * z.y;
-      acc[1] += rr[u].x * z.y + rr[u].y * z.x;
-      acc[2] += rr[u].x * rr[u].x + rr[u].y * rr[u].y;
+      sum[0].add(rr[u].x * z.x - rr[u].y * z.y);
+      sum[1].add(rr[u].x * z.y + rr[u].y * z.x);
+      sum[2].add(rr[u].x * rr[u].x + rr[u].y * rr[u].y);
     }
   }
+  T acc[3] = {sum[0].value(), sum[1].value(), sum[2].value()};
   fit_block_sum<T, 3>(acc, part + PSLOT(p, b));
   last_block_fin<3>(part, cnt, sys, p, b, OpCocgRho{});
 }
@@ -1093,8 +1115,10 @@ __global__ void __launch_bounds__(256) k_fg_givens(const double* __restrict__ pa
 // whole share of the elements, and nothing is exchanged between threads until the end.  The passes are
 // HBM-bound then (a few FMAs per 8 bytes), with NV independent coalesced loads in flight per thread; mode
 // 1 keeps the NV values of its element for the dot products (NV <= 32), so V is read once.  Sums run in
-// FP32 over a thread's elements and a warp's shuffles and in FP64 from there on.  NV is nv rounded up to
+// FP32 over FG_RUN of a thread's elements and a warp's shuffles and in FP64 from there on, so that their rounding
+// depends neither on the size of the grid nor on the batch.  NV is nv rounded up to
 // a multiple of 4; blocks of 128 threads, as many per SM as the registers of the mode allow.
+constexpr int FG_RUN = 8;
 template <int NV, int MODE>
 __host__ __device__ constexpr int fg_blocks_per_sm() {
   return NV <= 8 ? 8 : (NV <= 16 ? (MODE == 1 ? 4 : 5) : (NV <= 32 ? (NV <= 24 ? (MODE == 1 ? 3 : 4) : (MODE == 1 ? 2 : 3)) : 2));
@@ -1131,7 +1155,7 @@ __global__ void __launch_bounds__(128, (fg_blocks_per_sm<NV, MODE>())) k_fg_stre
   const int b = blockIdx.y;
   if (sys[b].inner_status != SYS_RUN) return;
   __shared__ float2 hs[NV];
-  __shared__ float red[4][2 * NV];
+  __shared__ double wsum[4][2 * NV];  // per warp
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const long long vs = (long long)p.B * p.ne, off = (long long)b * p.ne;
   const float2* v0 = Vb + off;
@@ -1143,64 +1167,71 @@ __global__ void __launch_bounds__(128, (fg_blocks_per_sm<NV, MODE>())) k_fg_stre
                      : make_float2(0.f, 0.f);
     __syncthreads();
   }
+  for (int q = lane; q < 2 * NV; q += 32) wsum[warp][q] = 0.0;
+  __syncwarp();
   float ar[NV], ai[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) ar[i] = ai[i] = 0.f;
-  for (long long e = blockIdx.x * 128LL + tid; e < p.ne; e += (long long)gridDim.x * 128) {
-    // (the vectors' addresses by repeated addition: as i * vs the compiler keeps 2 NV registers of offsets)
-    const float2* ve = v0 + e;
-    float2 wv = w[e];
-    float2 a[KEEP ? NV : 1];
-    if (KEEP) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) {
-        a[KEEP ? i : 0] = i < nv ? *ve : make_float2(0.f, 0.f);
-        ve += vs;
-      }
-    }
-    if (MODE == 1) {
+  long long e = blockIdx.x * 128LL + tid;
+  while (__any_sync(0xffffffffu, e < p.ne)) {
+    for (int run = 0; run < FG_RUN && e < p.ne; ++run, e += (long long)gridDim.x * 128) {
+      // (the vectors' addresses by repeated addition: as i * vs the compiler keeps 2 NV registers of offsets)
+      const float2* ve = v0 + e;
+      float2 wv = w[e];
+      float2 a[KEEP ? NV : 1];
       if (KEEP) {
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-          const float2 h = hs[i], c = a[KEEP ? i : 0];
-          wv.x -= h.x * c.x - h.y * c.y;
-          wv.y -= h.x * c.y + h.y * c.x;
+          a[KEEP ? i : 0] = i < nv ? *ve : make_float2(0.f, 0.f);
+          ve += vs;
         }
-      } else {
-        const float2* vi = ve;
+      }
+      if (MODE == 1) {
+        if (KEEP) {
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            const float2 h = hs[i], c = a[KEEP ? i : 0];
+            wv.x -= h.x * c.x - h.y * c.y;
+            wv.y -= h.x * c.y + h.y * c.x;
+          }
+        } else {
+          const float2* vi = ve;
 #pragma unroll 8
-        for (int i = 0; i < nv; ++i) {
-          const float2 h = hs[i], c = *vi;
-          wv.x -= h.x * c.x - h.y * c.y;
-          wv.y -= h.x * c.y + h.y * c.x;
-          vi += vs;
+          for (int i = 0; i < nv; ++i) {
+            const float2 h = hs[i], c = *vi;
+            wv.x -= h.x * c.x - h.y * c.y;
+            wv.y -= h.x * c.y + h.y * c.x;
+            vi += vs;
+          }
         }
+        w[e] = wv;
       }
-      w[e] = wv;
-    }
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      float2 c;
-      if (KEEP) {
-        c = a[KEEP ? i : 0];
-      } else {
-        c = i < nv ? *ve : make_float2(0.f, 0.f);
-        ve += vs;
+      for (int i = 0; i < NV; ++i) {
+        float2 c;
+        if (KEEP) {
+          c = a[KEEP ? i : 0];
+        } else {
+          c = i < nv ? *ve : make_float2(0.f, 0.f);
+          ve += vs;
+        }
+        ar[i] += c.x * wv.x + c.y * wv.y;  // conj(V_i) w
+        ai[i] += c.x * wv.y - c.y * wv.x;
       }
-      ar[i] += c.x * wv.x + c.y * wv.y;  // conj(V_i) w
-      ai[i] += c.x * wv.y - c.y * wv.x;
     }
-  }
+    __syncwarp();
 #pragma unroll
-  for (int i = 0; i < NV; i += 4) {
-    float v[8] = {ar[i], ai[i], ar[i + 1], ai[i + 1], ar[i + 2], ai[i + 2], ar[i + 3], ai[i + 3]};
-    int which;
-    const float t = warp_sum8(v, lane, &which);
-    if ((lane & 3) == 0) red[warp][2 * i + which] = t;
+    for (int i = 0; i < NV; i += 4) {
+      float v[8] = {ar[i], ai[i], ar[i + 1], ai[i + 1], ar[i + 2], ai[i + 2], ar[i + 3], ai[i + 3]};
+      int which;
+      const float t = warp_sum8(v, lane, &which);
+      if ((lane & 3) == 0) wsum[warp][2 * i + which] += (double)t;  // (always the same lane's)
+      ar[i] = ai[i] = ar[i + 1] = ai[i + 1] = ar[i + 2] = ai[i + 2] = ar[i + 3] = ai[i + 3] = 0.f;
+    }
   }
   __syncthreads();
   for (int q = tid; q < 2 * nv; q += 128)
-    *fg_slot(part, p, b, q) = ((double)red[0][q] + (double)red[1][q]) + ((double)red[2][q] + (double)red[3][q]);
+    *fg_slot(part, p, b, q) = (wsum[0][q] + wsum[1][q]) + (wsum[2][q] + wsum[3][q]);
 }
 
 // mode 2, complex64: the update streams the vectors eight at a time (no sums to keep)
@@ -1218,7 +1249,7 @@ __global__ void __launch_bounds__(256, 5) k_fg_stream_norm(const float2* __restr
                    : make_float2(0.f, 0.f);
   __syncthreads();
   w += off;
-  float nrm[1] = {0.f};
+  RunSum<float> sum;
   for (long long e = blockIdx.x * 256LL + tid; e < p.ne; e += (long long)gridDim.x * 256) {
     const float2* ve = Vb + off + e;
     float2 wv = w[e];
@@ -1237,8 +1268,9 @@ __global__ void __launch_bounds__(256, 5) k_fg_stream_norm(const float2* __restr
       }
     }
     w[e] = wv;
-    nrm[0] += wv.x * wv.x + wv.y * wv.y;
+    sum.add(wv.x * wv.x + wv.y * wv.y);
   }
+  float nrm[1] = {sum.value()};
   fit_block_sum<float, 1>(nrm, fg_slot(part, p, b, 0));
 }
 
