@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "fit_internal.cuh"
+#include "fit_residency.cuh"
 
 namespace {
 
@@ -1791,14 +1792,17 @@ struct Seq {
     (void)cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
     check();
   }
-  // grid of an iteration's vector pass: a few blocks per SM shared by the batch.  One large complex64 system
-  // wants more bytes in flight (4: 127.8, 6: 126.9, 8: 130.2 us per COCG iteration at 128^3); small batches and
-  // complex128 fewer partial sums in FP64 (8 x 40x36x28: 4: 62.0, 6: 64.3; complex128 4: 139.7, 8: 147.8).
+  // grid of an iteration's vector pass: a few blocks per SM shared by the batch.  One complex64 system wants
+  // more bytes in flight (128^3, us per COCG iteration: 4: 127.8, 6: 126.9, 8: 130.2); batches and complex128
+  // fewer partial sums in FP64 (8 x 40x36x28: 4: 62.0, 6: 64.3; complex128 4: 139.7, 8: 147.8).  No system gets
+  // less than a quarter of the SMs: blocks of systems that have finished leave at once, and the last ones of a
+  // sweep would run on a few SMs (64 x 40x36x28 from 0.5 to 20 GHz, COCG: 9 blocks 123.0 us per iteration, 38: 117.0,
+  // 76: 114.6, 152: 128.3; 16 systems: 38: 47.7, 76: 49.6, 152: 51.1).
   dim3 igrid() const {
     const int per_sm = w.mixed && w.p.B == 1 ? 6 : 4;
     const long long fill = (w.p.ne + 255) / 256;
-    const long long n = std::max(1LL, (long long)per_sm * w.nsm / w.p.B);
-    return dim3((unsigned)std::max(1LL, std::min({n, fill, (long long)w.p.nblk})), w.p.B);
+    return dim3((unsigned)fit_blocks_per_system(per_sm, w.nsm, w.p.B, w.nsm / 4, std::min(fill, (long long)w.p.nblk)),
+                w.p.B);
   }
   template <int NQ, class Op>
   void fin(const double* part, long long nslots, int stride, Op op) {
@@ -1948,12 +1952,13 @@ struct Seq {
     check();
     ortho_fin<MODE>(j, w.p.nblk);
   }
-  // blocks per system of a streaming pass: the resident blocks shared by the batch, no more than the elements
-  // fill and no more than the partial-sum buffer holds
+  // blocks per system of a streaming pass: the resident blocks shared by the batch but no fewer than the SMs
+  // (systems that have finished leave theirs idle: FGMRES(30), 40x36x28 from 0.5 to 20 GHz, us per step: 16 systems
+  // 118.3 without the lower limit, 98.7 with it; 64 systems 368.3 and 230.8), no more than the elements fill and no
+  // more than the partial-sum buffer holds
   int stream_blocks(int per_sm, int threads) const {
     const long long fill = (w.p.ne + threads - 1) / threads;
-    const long long res = std::max(1LL, (long long)per_sm * w.nsm / w.p.B);
-    return (int)std::max(1LL, std::min({fill, res, (long long)w.p.nblk}));
+    return (int)fit_blocks_per_system(per_sm, w.nsm, w.p.B, w.nsm, std::min(fill, (long long)w.p.nblk));
   }
   template <int NV, int MODE>
   void ortho_stream(int nv, const double* h) {

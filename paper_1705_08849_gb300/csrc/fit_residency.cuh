@@ -1,14 +1,16 @@
-// What a launcher needs to know about a kernel on the current device, looked up once per kernel and device: the
-// opt-in to its dynamic shared memory, which is an attribute of the kernel on one device, and the CTAs resident at
-// once.  (The runtime queries cost more than the launch of a small grid.)  Host code only.
+// Launch sizes.  Host code only.
 #pragma once
 
 #include <cuda_runtime_api.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <utility>
 
+// What a launcher needs to know about a kernel on the current device, looked up once per kernel and device: the
+// opt-in to its dynamic shared memory, which is an attribute of the kernel on one device, and the CTAs resident at
+// once.  (The runtime queries cost more than the launch of a small grid.)
 struct FitResidency {
   int per_sm = 0;  // CTAs per SM (0: not even one fits)
   int nsm = 0;     // SMs of the device
@@ -55,4 +57,11 @@ inline cudaError_t fit_residency(const void* kern, int threads, int smem, FitRes
         return cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(per_sm, kern, threads, smem, cudaOccupancyDefault);
       },
       out);
+}
+
+// Blocks that each system of a batch gets in a pass over all of them: per_sm blocks per SM shared by the batch, but at
+// least `least` for every system (those of systems that have finished leave at once, and must not be all that the
+// last ones have), and at most `most` (what the elements fill, what the pass's buffers hold).
+inline long long fit_blocks_per_system(int per_sm, int nsm, int batch, int least, long long most) {
+  return std::max(1LL, std::min(std::max((long long)least, (long long)per_sm * nsm / batch), most));
 }
