@@ -268,7 +268,7 @@ def _call_apply(call, what, g, ne, omega, x, y, prec, stream):
     grid's sizes, pointer objects and an import each)."""
     if type(omega) is not np.ndarray or omega.dtype != np.float64 or omega.ndim != 1 or not omega.flags.c_contiguous:
         omega = np.ascontiguousarray(np.atleast_1d(np.asarray(omega, dtype=np.float64)))
-    nb = omega.size
+    nb = len(omega)
     if ne is None:
         out = _Info()
         _check(lib().fit_grid_info(g, out), "fit_grid_info")
