@@ -281,9 +281,9 @@ static fit_status conv3_tc(const unet::ConvArgs& a, int cin, cudaStream_t s, boo
 // Weight gradient of a 3x3x3 conv on the tensor cores: dw (27 x cout x cin) and db accumulate (the caller
 // zeroes them).  One wave of resident blocks, a third of them for each z-tap, every one with about three row
 // segments' worth of y-chunks (at least eight rows each, so that a chunk's two halo rows stay a small part).
-template <int CO, int CI, int TV>
+template <int CO, int CI, int TV, bool ENDS>
 fit_status wgrad_launch_shape(const unet::WgradArgs& w, cudaStream_t s) {
-  auto kern = unet::conv3_wgrad_kernel<CO, CI, TV>;
+  auto kern = unet::conv3_wgrad_kernel<CO, CI, TV, ENDS>;
   constexpr int smem = unet::WgradShape<CO, CI>::smem(TV);
   FitResidency res;
   FIT_CHECK_CUDA(fit_residency((const void*)kern, 256, smem, &res));
@@ -307,12 +307,17 @@ fit_status wgrad_launch_shape(const unet::WgradArgs& w, cudaStream_t s) {
   return FIT_OK;
 }
 
+template <int CO, int CI, int TV>
+fit_status wgrad_launch_ends(const unet::WgradArgs& w, cudaStream_t s) {
+  return w.nx % TV ? wgrad_launch_shape<CO, CI, TV, true>(w, s) : wgrad_launch_shape<CO, CI, TV, false>(w, s);
+}
+
 fit_status wgrad_launch(const unet::WgradArgs& w, cudaStream_t s) {
   const int ci = w.c1 + w.c2, co = w.cout;
   // segments of 64 voxels, of 32 where a row has no more (half of a longer one would be padding)
 #define FIT_WG(CO_, CI_) \
   if (co == CO_ && ci == CI_) \
-    return w.nx <= 32 ? wgrad_launch_shape<CO_, CI_, 32>(w, s) : wgrad_launch_shape<CO_, CI_, 64>(w, s)
+    return w.nx <= 32 ? wgrad_launch_ends<CO_, CI_, 32>(w, s) : wgrad_launch_ends<CO_, CI_, 64>(w, s)
   FIT_WG(16, 16);
   FIT_WG(32, 16);
   FIT_WG(32, 32);

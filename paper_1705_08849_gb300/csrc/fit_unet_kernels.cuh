@@ -4,6 +4,8 @@
 // voxel index x + nx*(y + ny*z)).
 #pragma once
 
+#include <type_traits>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -624,6 +626,10 @@ struct WgradShape {
   static constexpr int MT = CO / 16, NT = CI / 8, COMBOS = MT * NT;
   static constexpr int WT = COMBOS >= 16 ? 8 : (COMBOS >= 4 ? 4 : 2), WK = 8 / WT;
   static constexpr int NCB = COMBOS / WT;  // 8-channel columns per warp, all of one 16-row group
+  // Blocks per SM that the registers must leave room for (36 NCB accumulators per thread; 0: the compiler's choice).
+  // ENDS: the second pass, compiled with the first, would otherwise cost every call a block (32 -> 32 at nx = 65: 94 us
+  // for 62).  NCB = 4: there is no second block to save registers for (64 -> 64 at nx = 64: 128 -> 112 us).
+  static constexpr int blocks(bool ends) { return NCB == 4 ? 1 : (!ends ? 0 : (NCB == 1 ? 3 : 2)); }
   static constexpr int RSO = CO + 8, RSI = CI + 8;  // padded row strides (conflict-free ldmatrix)
   static constexpr int XR = 8, YR = 4;              // rings: rows of X and of dY
   static constexpr int stage_bytes(int TV) { return (XR * (TV + 2) * RSI + YR * TV * RSO) * 2; }
@@ -633,8 +639,12 @@ struct WgradShape {
   }
 };
 
-template <int CO, int CI, int TV>
-__global__ void __launch_bounds__(256) conv3_wgrad_kernel(WgradArgs a, int ylen, int nyc, int ntask) {
+// ENDS: rows end inside their last segment (nx is no multiple of TV).  The first voxel past the end has no dY (zero),
+// but the taps at x - 1 find the row's last voxel there, and zero times an infinite or NaN one is NaN.  A block whose
+// sums of those taps are not finite goes over its segments once more and clears that voxel from their X fragments.
+// (Clearing it in the first pass costs every call 4 to 15%.)
+template <int CO, int CI, int TV, bool ENDS>
+__global__ void __launch_bounds__(256, (WgradShape<CO, CI>::blocks(ENDS))) conv3_wgrad_kernel(WgradArgs a, int ylen, int nyc, int ntask) {
   using SH = WgradShape<CO, CI>;
   constexpr int RSO = SH::RSO, RSI = SH::RSI, NCB = SH::NCB, WK = SH::WK, XR = SH::XR, YR = SH::YR;
   constexpr int KS = TV / 16;
@@ -649,112 +659,134 @@ __global__ void __launch_bounds__(256) conv3_wgrad_kernel(WgradArgs a, int ylen,
   const int q = lane >> 3, r = lane & 7;  // ldmatrix: which 8x8 matrix this lane addresses, and its row
   const int nseg = (a.nx + TV - 1) / TV;
   float acc[9][NCB][4];
-#pragma unroll
-  for (int t = 0; t < 9; ++t)
-#pragma unroll
-    for (int n = 0; n < NCB; ++n)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[t][n][c] = 0.f;
   float dbs = 0.f;  // dz = 1: this thread's share of db[tid % CO]
-  for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
-    const int xs = (task % nseg) * TV, yc = (task / nseg) % nyc, z = task / (nseg * nyc);
-    const int zx = z + dz - 1;
-    if (zx < 0 || zx >= a.nz) continue;  // (dz = 1 never is: db misses nothing)
-    const int y0 = yc * ylen, y1 = min(a.ny, y0 + ylen);
-    auto load_x = [&](int y) {  // row y of the plane zx, voxels xs-1 .. xs+TV
-      bf16* dst = sx + ((y + 1) & (XR - 1)) * (TV + 2) * RSI;
-      const bool yin = y >= 0 && y < a.ny;
-      const long long row = (long long)a.nx * (y + (long long)a.ny * zx);
-      for (int e = tid; e < (TV + 2) * (CI / 8); e += 256) {
-        const int v = e / (CI / 8), c = (e % (CI / 8)) * 8, gx = xs - 1 + v;
-        const bool in = yin && gx >= 0 && gx < a.nx;
-        const bf16* src = a.dy;  // a valid address even when nothing is read
-        if (in) src = c < a.c1 ? a.x1 + (row + gx) * a.c1 + c : a.x2 + (row + gx) * a.c2 + (c - a.c1);
-        cp_async16(smem_addr(dst + v * RSI + c), src, in ? 16 : 0);
-      }
-    };
-    auto load_dy = [&](int y) {
-      bf16* dst = sdy + (y & (YR - 1)) * TV * RSO;
-      const long long row = (long long)a.nx * (y + (long long)a.ny * z);
-      for (int e = tid; e < TV * (CO / 8); e += 256) {
-        const int v = e / (CO / 8), c = (e % (CO / 8)) * 8;
-        const bool in = y < y1 && xs + v < a.nx;
-        cp_async16(smem_addr(dst + v * RSO + c), in ? a.dy + (row + xs + v) * CO + c : a.dy, in ? 16 : 0);
-      }
-    };
-    __syncthreads();  // the previous segment's rows are read
-    load_x(y0 - 1);
-    load_x(y0);
-    load_x(y0 + 1);
-    load_dy(y0);
-    cp_async_commit();
-    load_x(y0 + 2);
-    load_dy(y0 + 1);
-    cp_async_commit();
-    for (int y = y0; y < y1; ++y) {
-      if (y + 2 < y1) {  // the rows of step y + 2
-        load_x(y + 3);
-        load_dy(y + 2);
-      }
-      cp_async_commit();  // (possibly empty)
-      cp_async_wait<2>();
-      __syncthreads();
-      const bf16* dyr = sdy + (y & (YR - 1)) * TV * RSO;
-      if (a.db && dz == 1)
-        for (int v = tid / CO; v < TV; v += 256 / CO) dbs += __bfloat162float(dyr[v * RSO + tid % CO]);
-      auto load_a = [&](int kk, uint32_t (&f)[4]) {
-        ldsm_x4_t(smem_addr(dyr + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), f[0], f[1], f[2], f[3]);
+  auto all_segments = [&](auto cut) {  // cut: clear the voxels past the row ends
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+#pragma unroll
+      for (int n = 0; n < NCB; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[t][n][c] = 0.f;
+    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+      const int xs = (task % nseg) * TV, yc = (task / nseg) % nyc, z = task / (nseg * nyc);
+      const int zx = z + dz - 1;
+      if (zx < 0 || zx >= a.nz) continue;  // (dz = 1 never is: db misses nothing)
+      const int y0 = yc * ylen, y1 = min(a.ny, y0 + ylen);
+      // the 16-voxel step and half fragment of the first voxel past the end; voxel 2 (lane % 4) + h of a fragment's 8
+      // sits in half h of the lane's register
+      const int vend = a.nx - xs, kend = cut && vend < TV ? vend >> 4 : -1;
+      uint32_t keep[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
+      if (cut && (lane & 3) == ((vend & 7) >> 1)) keep[(vend >> 3) & 1] = vend & 1 ? 0x0000FFFFu : 0xFFFF0000u;
+      auto load_x = [&](int y) {  // row y of the plane zx, voxels xs-1 .. xs+TV
+        bf16* dst = sx + ((y + 1) & (XR - 1)) * (TV + 2) * RSI;
+        const bool yin = y >= 0 && y < a.ny;
+        const long long row = (long long)a.nx * (y + (long long)a.ny * zx);
+        for (int e = tid; e < (TV + 2) * (CI / 8); e += 256) {
+          const int v = e / (CI / 8), c = (e % (CI / 8)) * 8, gx = xs - 1 + v;
+          const bool in = yin && gx >= 0 && gx < a.nx;
+          const bf16* src = a.dy;  // a valid address even when nothing is read
+          if (in) src = c < a.c1 ? a.x1 + (row + gx) * a.c1 + c : a.x2 + (row + gx) * a.c2 + (c - a.c1);
+          cp_async16(smem_addr(dst + v * RSI + c), src, in ? 16 : 0);
+        }
       };
-      auto xrow = [&](int t, int kk) {
-        return sx + ((y + t / 3) & (XR - 1)) * (TV + 2) * RSI + (kk + t % 3) * RSI + nt0 * 8;
+      auto load_dy = [&](int y) {
+        bf16* dst = sdy + (y & (YR - 1)) * TV * RSO;
+        const long long row = (long long)a.nx * (y + (long long)a.ny * z);
+        for (int e = tid; e < TV * (CO / 8); e += 256) {
+          const int v = e / (CO / 8), c = (e % (CO / 8)) * 8;
+          const bool in = y < y1 && xs + v < a.nx;
+          cp_async16(smem_addr(dst + v * RSO + c), in ? a.dy + (row + xs + v) * CO + c : a.dy, in ? 16 : 0);
+        }
       };
-      if constexpr (NCB > 1) {  // two 8-channel columns per fragment load
+      __syncthreads();  // the previous segment's rows are read
+      load_x(y0 - 1);
+      load_x(y0);
+      load_x(y0 + 1);
+      load_dy(y0);
+      cp_async_commit();
+      load_x(y0 + 2);
+      load_dy(y0 + 1);
+      cp_async_commit();
+      for (int y = y0; y < y1; ++y) {
+        if (y + 2 < y1) {  // the rows of step y + 2
+          load_x(y + 3);
+          load_dy(y + 2);
+        }
+        cp_async_commit();  // (possibly empty)
+        cp_async_wait<2>();
+        __syncthreads();
+        const bf16* dyr = sdy + (y & (YR - 1)) * TV * RSO;
+        if (!cut && a.db && dz == 1)
+          for (int v = tid / CO; v < TV; v += 256 / CO) dbs += __bfloat162float(dyr[v * RSO + tid % CO]);
+        auto load_a = [&](int kk, uint32_t (&f)[4]) {
+          ldsm_x4_t(smem_addr(dyr + (kk + (q >> 1) * 8 + r) * RSO + mt * 16 + (q & 1) * 8), f[0], f[1], f[2], f[3]);
+        };
+        auto xrow = [&](int t, int kk) {
+          return sx + ((y + t / 3) & (XR - 1)) * (TV + 2) * RSI + (kk + t % 3) * RSI + nt0 * 8;
+        };
+        if constexpr (NCB > 1) {  // two 8-channel columns per fragment load
 #pragma unroll
-        for (int k = wk; k < KS; k += WK) {
-          uint32_t fa[4];
-          load_a(k * 16, fa);
+          for (int k = wk; k < KS; k += WK) {
+            uint32_t fa[4];
+            load_a(k * 16, fa);
 #pragma unroll
-          for (int t = 0; t < 9; ++t) {
-            const bf16* xr = xrow(t, k * 16);
+            for (int t = 0; t < 9; ++t) {
+              const bf16* xr = xrow(t, k * 16);
 #pragma unroll
-            for (int n = 0; n < NCB; n += 2) {
+              for (int n = 0; n < NCB; n += 2) {
+                uint32_t b0, b1, b2, b3;
+                ldsm_x4_t(smem_addr(xr + ((q & 1) * 8 + r) * RSI + n * 8 + (q >> 1) * 8), b0, b1, b2, b3);
+                if (cut && t % 3 == 0 && k == kend) b0 &= keep[0], b1 &= keep[1], b2 &= keep[0], b3 &= keep[1];
+                mma_bf16(acc[t][n], fa[0], fa[1], fa[2], fa[3], b0, b1);
+                mma_bf16(acc[t][n + 1], fa[0], fa[1], fa[2], fa[3], b2, b3);
+              }
+            }
+          }
+        } else if constexpr (KS >= 2 * WK) {  // one column: two of the warp's 16-voxel steps per load
+#pragma unroll
+          for (int k = wk; k < KS; k += 2 * WK) {
+            uint32_t fa[4], fb[4];
+            load_a(k * 16, fa);
+            load_a((k + WK) * 16, fb);
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
               uint32_t b0, b1, b2, b3;
-              ldsm_x4_t(smem_addr(xr + ((q & 1) * 8 + r) * RSI + n * 8 + (q >> 1) * 8), b0, b1, b2, b3);
-              mma_bf16(acc[t][n], fa[0], fa[1], fa[2], fa[3], b0, b1);
-              mma_bf16(acc[t][n + 1], fa[0], fa[1], fa[2], fa[3], b2, b3);
+              ldsm_x4_t(smem_addr(xrow(t, (k + (q >> 1) * WK) * 16) + ((q & 1) * 8 + r) * RSI), b0, b1, b2, b3);
+              if (cut && t % 3 == 0 && k == kend) b0 &= keep[0], b1 &= keep[1];
+              if (cut && t % 3 == 0 && k + WK == kend) b2 &= keep[0], b3 &= keep[1];
+              mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
+              mma_bf16(acc[t][0], fb[0], fb[1], fb[2], fb[3], b2, b3);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int k = wk; k < KS; k += WK) {
+            uint32_t fa[4];
+            load_a(k * 16, fa);
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+              uint32_t b0, b1;
+              ldsm_x2_t(smem_addr(xrow(t, k * 16) + (lane & 15) * RSI), b0, b1);
+              if (cut && t % 3 == 0 && k == kend) b0 &= keep[0], b1 &= keep[1];
+              mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
             }
           }
         }
-      } else if constexpr (KS >= 2 * WK) {  // one column: two of the warp's 16-voxel steps per load
-#pragma unroll
-        for (int k = wk; k < KS; k += 2 * WK) {
-          uint32_t fa[4], fb[4];
-          load_a(k * 16, fa);
-          load_a((k + WK) * 16, fb);
-#pragma unroll
-          for (int t = 0; t < 9; ++t) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4_t(smem_addr(xrow(t, (k + (q >> 1) * WK) * 16) + ((q & 1) * 8 + r) * RSI), b0, b1, b2, b3);
-            mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
-            mma_bf16(acc[t][0], fb[0], fb[1], fb[2], fb[3], b2, b3);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int k = wk; k < KS; k += WK) {
-          uint32_t fa[4];
-          load_a(k * 16, fa);
-#pragma unroll
-          for (int t = 0; t < 9; ++t) {
-            uint32_t b0, b1;
-            ldsm_x2_t(smem_addr(xrow(t, k * 16) + (lane & 15) * RSI), b0, b1);
-            mma_bf16(acc[t][0], fa[0], fa[1], fa[2], fa[3], b0, b1);
-          }
-        }
+        __syncthreads();  // row y - 1 of X and row y of dY are refilled two steps on
       }
-      __syncthreads();  // row y - 1 of X and row y of dY are refilled two steps on
+      cp_async_wait<0>();
     }
-    cp_async_wait<0>();
+  };
+  all_segments(std::false_type{});
+  if constexpr (ENDS) {
+    float worst = 0.f;  // (0 times anything that is not finite is NaN)
+#pragma unroll
+    for (int t = 0; t < 9; t += 3)
+#pragma unroll
+      for (int n = 0; n < NCB; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) worst = fmaf(acc[t][n][c], 0.f, worst);
+    if (__syncthreads_or(worst != 0.f)) all_segments(std::true_type{});
   }
   const int cin = a.c1 + a.c2;
   float* dw = a.dw + (long long)dz * 9 * CO * cin;
