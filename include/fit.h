@@ -253,7 +253,8 @@ fit_status fit_set_hbm_budget(fit_grid* g, size_t bytes);
 fit_status fit_grid_info(const fit_grid* g, long long* out6);
 
 /* fit_apply_variant_count -- number of launch shapes of the fused TMA stencil kernel for a precision
- * (the candidates the autotuner times; see fit_apply_tuned). */
+ * (the candidates the autotuner times; see fit_apply_tuned).  complex64 grids with an odd nx run the
+ * warp-specialised ones only, and the generic kernel where another is asked for. */
 int fit_apply_variant_count(fit_prec prec);
 
 /* fit_apply_tuned -- the apply kernel the autotuner picked for (prec, nbatch) on this grid:
@@ -272,11 +273,12 @@ int fit_apply_variant_count(fit_prec prec);
  * Candidates are timed from a cold L2: for the duration of the tuning the handle holds a scratch
  * buffer of twice the L2 size (counted against fit_set_hbm_budget; if it does not fit, candidates
  * are timed back to back instead).
+ * complex64 grids with an odd nx are not timed: their shape follows from the grid and the batch by rule.
  * Tests and experiments can force a kernel with the environment variable
  * FIT_APPLY_KERNEL=generic or FIT_APPLY_KERNEL=fused:<k>.
- * Persistence (opt-in): with FIT_TUNE_CACHE=<file> set, the autotuner first looks the key up in that
- * file (fit_tuning_lookup) and uses a recorded choice without timing anything; after a search it
- * appends its result (fit_tuning_record).  The key is the device name and SM count, the grid size, the
+ * Persistence (opt-in): with FIT_TUNE_CACHE=<file> set, the first call first looks the key up in that
+ * file (fit_tuning_lookup) and uses a recorded choice without timing anything; after a search (not for a
+ * choice by rule) it appends its result (fit_tuning_record).  The key is the device name and SM count, the grid size, the
  * precision and the batch. */
 fit_status fit_apply_tuned(const fit_grid* g, fit_prec prec, int nbatch, int* out7);
 

@@ -1671,12 +1671,8 @@ fit_status fit_tune_apply(fit_grid* g, int nbatch, const fit_omega& om, const vo
     g->tuned[key] = -1;
     return FIT_OK;
   }
-  if (prec == FIT_C64 && g->nx % 2 != 0) {  // (no search: see odd_choice)
-    g->tuned[key] = odd_choice(g, nbatch);
-    return FIT_OK;
-  }
   // opt-in persistence: a cache file named by FIT_TUNE_CACHE supplies the choice for this device, grid,
-  // precision and batch if it holds one, and records the result of a new search
+  // precision and batch if it holds one, and records the result of a search
   const char* cache = getenv("FIT_TUNE_CACHE");
   std::string dev_name;
   int sms = 0;
@@ -1687,6 +1683,10 @@ fit_status fit_tune_apply(fit_grid* g, int nbatch, const fit_omega& om, const vo
       g->tuned[key] = c;
       return FIT_OK;
     }
+  }
+  if (prec == FIT_C64 && g->nx % 2 != 0) {  // (no search: see odd_choice)
+    g->tuned[key] = odd_choice(g, nbatch);
+    return FIT_OK;
   }
   int n = 0;
   const Variant* vars = variants(prec, &n);
