@@ -47,22 +47,21 @@ namespace {
 
 constexpr int TX = 32;  // one warp per tile row
 
-template <typename T, int TY, bool KU = false>  // KU: the stage also holds the epilogue vector u
+template <int TY, bool KU = false>  // KU: the stage also holds the epilogue vector u
 struct Layout {
-  using V = typename cplx<T>::t;
-  static constexpr int CE = sizeof(V) / 8;      // 8-byte copy elements per complex value
+  using V = float2;
   static constexpr int EW = 3 * (TX + 4);       // complex values per staged e row
   static constexpr int ER = TY + 2;
-  static constexpr int NW = 3 * (TX + 4);       // T values per staged M_nu row
+  static constexpr int NW = 3 * (TX + 4);       // values per staged M_nu row
   static constexpr int NR = TY + 1;
-  static constexpr int KW = 6 * TX;             // T values per staged M_eps/M_kappa row
+  static constexpr int KW = 6 * TX;             // values per staged M_eps/M_kappa row
   static constexpr int MW = TX + 32;            // mask bytes per staged row
   static constexpr int MR = TY + 2;
   static constexpr int OW = 3 * TX;             // complex values per output / u row
   static constexpr int al(int b) { return (b + 127) / 128 * 128; }
   static constexpr int E_BYTES = EW * ER * (int)sizeof(V);
-  static constexpr int N_BYTES = NW * NR * (int)sizeof(T);
-  static constexpr int K_BYTES = KW * TY * (int)sizeof(T);
+  static constexpr int N_BYTES = NW * NR * (int)sizeof(float);
+  static constexpr int K_BYTES = KW * TY * (int)sizeof(float);
   static constexpr int M_BYTES = MW * MR;
   static constexpr int U_BYTES = OW * TY * (int)sizeof(V);  // also the size of one output buffer
   static constexpr int E_OFF = 0;
@@ -221,17 +220,18 @@ __device__ inline void programmatic_start() {
 // Persistent: the grid holds one wave of CTAs; CTA c processes tiles c, c + gridDim.x, ...
 // (tile = x-tile, y-tile, z-chunk, system; x fastest).  The plane counter G and the output counter
 // O run across tiles, so ring-stage parities and output buffers stay consistent.
-template <typename T, int TY, int EPI, int S>
+template <int TY, int EPI, int S>
 __global__ void __launch_bounds__(TX* TY, TY == 4 ? 5 : (TY == 8 ? 3 : 1)) fused_apply_kernel(const __grid_constant__ CUtensorMap tm_x,
                                                                 const __grid_constant__ CUtensorMap tm_y,
                                                                 const __grid_constant__ CUtensorMap tm_u,
                                                                 const __grid_constant__ CUtensorMap tm_nu,
                                                                 const __grid_constant__ CUtensorMap tm_ek,
                                                                 const __grid_constant__ CUtensorMap tm_mask,
-                                                                const __grid_constant__ FusedArgs<T> a, fit_epi epi) {
-  using V = typename cplx<T>::t;
+                                                                const __grid_constant__ FusedArgs<float> a, fit_epi epi) {
+  using T = float;
+  using V = float2;
   constexpr bool kU = (EPI == FIT_EPI_DOT_U || EPI == FIT_EPI_RESID);
-  using L = Layout<T, TY, kU>;
+  using L = Layout<TY, kU>;
   constexpr uint32_t kTx = L::TX_BYTES + (kU ? L::U_BYTES : 0);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
@@ -270,20 +270,20 @@ __global__ void __launch_bounds__(TX* TY, TY == 4 ? 5 : (TY == 8 ? 3 : 1)) fused
       unsigned char* st = stage(G0 + q);
       uint64_t* bar = &bars[(G0 + q) % S];
       mbar_expect_tx(bar, kTx);
-      tma_load_4d(st + L::E_OFF, &tm_x, L::CE * 3 * (i0 - 2), j0 - 1, p, b, bar);
+      tma_load_4d(st + L::E_OFF, &tm_x, 3 * (i0 - 2), j0 - 1, p, b, bar);
       tma_load_3d(st + L::N_OFF, &tm_nu, 3 * (i0 - 4), j0 - 1, p, bar);
       tma_load_3d(st + L::K_OFF, &tm_ek, 6 * i0, j0, p, bar);
       tma_load_3d(st + L::M_OFF, &tm_mask, i0 - 16, j0 - 1, p, bar);
-      if (kU) tma_load_4d(st + L::U_OFF, &tm_u, L::CE * 3 * i0, j0, p, b, bar);
+      if (kU) tma_load_4d(st + L::U_OFF, &tm_u, 3 * i0, j0, p, b, bar);
     };
     auto prefetch = [&](int q) {  // thread 0 only: the boxes of plane q into L2
       if (q >= nplanes) return;
       const int p = k0 - 1 + q;
-      tma_prefetch_4d(&tm_x, L::CE * 3 * (i0 - 2), j0 - 1, p, b);
+      tma_prefetch_4d(&tm_x, 3 * (i0 - 2), j0 - 1, p, b);
       tma_prefetch_3d(&tm_nu, 3 * (i0 - 4), j0 - 1, p);
       tma_prefetch_3d(&tm_ek, 6 * i0, j0, p);
       tma_prefetch_3d(&tm_mask, i0 - 16, j0 - 1, p);
-      if (kU) tma_prefetch_4d(&tm_u, L::CE * 3 * i0, j0, p, b);
+      if (kU) tma_prefetch_4d(&tm_u, 3 * i0, j0, p, b);
     };
     auto wait = [&](int q) {
       if (!mbar_wait(&bars[(G0 + q) % S], ((G0 + q) / S) & 1, a.abort)) {
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(TX* TY, TY == 4 ? 5 : (TY == 8 ? 3 : 1)) fused
       if (bad) break;
       if (tid == 0) {
         if (pend) tma_store_4d(&tm_y, obuf + (size_t)((O - 1) & 1) * (L::O_BYTES / sizeof(V)),
-                               L::CE * 3 * pi0, pj0, pk, pb);
+                               3 * pi0, pj0, pk, pb);
         if (qk - 1 + S < nplanes) {
           issue(qk - 1 + S);  // plane qk-1 is released by the barrier above
           if (a.pf) prefetch(qk - 1 + S + a.pf);
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(TX* TY, TY == 4 ? 5 : (TY == 8 ? 3 : 1)) fused
     G += nplanes;
     __syncthreads();  // stages free for the next tile; the last output plane is staged
     if (tid == 0 && pend) tma_store_4d(&tm_y, obuf + (size_t)((O - 1) & 1) * (L::O_BYTES / sizeof(V)),
-                                       L::CE * 3 * pi0, pj0, pk, pb);
+                                       3 * pi0, pj0, pk, pb);
     pend = false;
     if (EPI != FIT_EPI_NONE) {
       const long long nblk = (long long)a.ntx * a.nty * a.nzc;
@@ -1227,126 +1227,6 @@ cudaLaunchConfig_t programmatic_config(int grid, dim3 block, int smem, cudaStrea
   return cfg;
 }
 
-template <typename T, int TY, int S>
-fit_status launch_variant(fit_grid* g, int nbatch, const fit_omega& om, const void* x, void* y, const T* nu,
-                          const T* ek, double out_scale, cudaStream_t s, fit_epi& e, int tz, int pf) {
-  const bool c64 = sizeof(T) == 4;
-  CUtensorMap mx, mnu, mek, mmask;
-  const cuuint64_t ce = c64 ? 1 : 2;
-  {
-    cuuint64_t dims[4] = {3 * ce * (cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, (cuuint64_t)nbatch};
-    cuuint64_t rowb = 3 * ce * 8 * (cuuint64_t)g->nx;
-    cuuint64_t str[3] = {rowb, rowb * g->ny, rowb * g->ny * g->nz};
-    cuuint32_t box[4] = {(cuuint32_t)(3 * ce * (TX + 4)), TY + 2, 1, 1};
-    if (!encode(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, x, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of x rejected");
-      return FIT_ECUDA;
-    }
-  }
-  const CUtensorMapDataType cdt = c64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-  {
-    cuuint64_t dims[3] = {3 * (cuuint64_t)g->nxp, (cuuint64_t)g->ny, (cuuint64_t)g->nz};
-    cuuint64_t rowb = 3 * sizeof(T) * (cuuint64_t)g->nxp;
-    cuuint64_t str[2] = {rowb, rowb * g->ny};
-    cuuint32_t box[3] = {3 * (TX + 4), TY + 1, 1};
-    if (!encode(&mnu, cdt, 3, nu, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of M_nu rejected");
-      return FIT_ECUDA;
-    }
-  }
-  {
-    cuuint64_t dims[3] = {6 * (cuuint64_t)g->nxp, (cuuint64_t)g->ny, (cuuint64_t)g->nz};
-    cuuint64_t rowb = 6 * sizeof(T) * (cuuint64_t)g->nxp;
-    cuuint64_t str[2] = {rowb, rowb * g->ny};
-    cuuint32_t box[3] = {6 * TX, TY, 1};
-    if (!encode(&mek, cdt, 3, ek, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of M_eps/M_kappa rejected");
-      return FIT_ECUDA;
-    }
-  }
-  {
-    cuuint64_t dims[3] = {(cuuint64_t)g->nxp, (cuuint64_t)g->ny, (cuuint64_t)g->nz};
-    cuuint64_t str[2] = {(cuuint64_t)g->nxp, (cuuint64_t)g->nxp * g->ny};
-    cuuint32_t box[3] = {TX + 32, TY + 2, 1};
-    if (!encode(&mmask, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, g->mask, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of the mask rejected");
-      return FIT_ECUDA;
-    }
-  }
-  // y (bulk tensor store, box of the own cells) and the epilogue vector u (same shape as x)
-  CUtensorMap my, mu;
-  {
-    cuuint64_t dims[4] = {3 * ce * (cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, (cuuint64_t)nbatch};
-    cuuint64_t rowb = 3 * ce * 8 * (cuuint64_t)g->nx;
-    cuuint64_t str[3] = {rowb, rowb * g->ny, rowb * g->ny * g->nz};
-    cuuint32_t box[4] = {(cuuint32_t)(3 * ce * TX), TY, 1, 1};
-    if (!encode(&my, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, y, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of y rejected");
-      return FIT_ECUDA;
-    }
-    const void* ub = (e.mode == FIT_EPI_DOT_U || e.mode == FIT_EPI_RESID) ? e.u : x;
-    if (((uintptr_t)ub & 15) != 0 || !encode(&mu, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, ub, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of the epilogue vector rejected");
-      return FIT_ECUDA;
-    }
-  }
-  FusedArgs<T> a;
-  a.x = (const typename cplx<T>::t*)x;
-  a.omega = om.dev;
-  for (int b = 0; b < FIT_OMEGA_ARGS; ++b) a.om[b] = !om.dev && b < nbatch ? om.host[b] : 0.0;
-  a.err = g->err_dev;
-  a.abort = g->abort_dev;
-  a.abort_first = g->abort_mirror;
-  a.nx = g->nx;
-  a.ny = g->ny;
-  a.nz = g->nz;
-  a.ntx = (g->nx + TX - 1) / TX;
-  a.nty = (g->ny + TY - 1) / TY;
-  a.ne = g->ne;
-  a.out_scale = (T)out_scale;
-  a.pf = pf;
-  a.flat = 0;
-  a.nb = nbatch;
-  dim3 block(TX, TY, 1);
-  const bool ku = e.mode == FIT_EPI_DOT_U || e.mode == FIT_EPI_RESID;
-  int smem = ku ? Layout<T, TY, true>::smem(S) : Layout<T, TY, false>::smem(S);
-  auto run = [&](auto kern) -> fit_status {
-    FitResidency res;
-    FIT_CHECK_CUDA(fit_residency((const void*)kern, (int)(block.x * block.y), smem, &res));
-    const long long slots = res.ctas();
-    if (slots < 1) {  // shared memory or registers do not allow one resident CTA of this shape
-      fit_set_error("fused apply: launch shape does not fit on an SM");
-      return FIT_EINVAL;
-    }
-    int grid = 0;
-    a.flat = 0;
-    int tzz = tz;
-    if (tzz <= 0) {  // balanced: as many equal z-chunks per column tile as the resident CTAs allow
-      const long long cols = (long long)a.ntx * a.nty * nbatch;
-      const long long per_col = std::max(1LL, slots / std::max(1LL, cols));
-      tzz = (int)std::max(2LL, ((long long)g->nz + per_col - 1) / per_col);
-    }
-    a.tz = tzz;
-    a.nzc = (g->nz + tzz - 1) / tzz;
-    a.ntiles = a.ntx * a.nty * a.nzc * nbatch;
-    e.nslots = (long long)a.ntx * a.nty * a.nzc;
-    grid = (int)std::max(1LL, std::min((long long)a.ntiles, slots));  // one persistent wave
-    cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = programmatic_config(grid, block, smem, s, at);
-    FIT_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, mx, my, mu, mnu, mek, mmask, a, e));
-    return FIT_OK;
-  };
-  switch (e.mode) {
-    case FIT_EPI_NONE: return run(fused_apply_kernel<T, TY, FIT_EPI_NONE, S>);
-    case FIT_EPI_DOT_U: return run(fused_apply_kernel<T, TY, FIT_EPI_DOT_U, S>);
-    case FIT_EPI_DOT_TS: return run(fused_apply_kernel<T, TY, FIT_EPI_DOT_TS, S>);
-    case FIT_EPI_RESID: return run(fused_apply_kernel<T, TY, FIT_EPI_RESID, S>);
-    case FIT_EPI_DOT_XY: return run(fused_apply_kernel<T, TY, FIT_EPI_DOT_XY, S>);
-  }
-  fit_set_error("fused apply: unknown epilogue");
-  return FIT_EINVAL;
-}
-
 // tensor maps of the padded coefficient arrays and the mask, boxes of a tile of TY rows
 template <typename T, int TY>
 fit_status encode_coefs(const fit_grid* g, const T* nu, const T* ek, CUtensorMap* mnu, CUtensorMap* mek,
@@ -1368,6 +1248,102 @@ fit_status encode_coefs(const fit_grid* g, const T* nu, const T* ek, CUtensorMap
   return FIT_OK;
 }
 
+// tensor map of a batch of complex vectors over the grid's cells, boxes of w x h cells of one plane
+template <typename T>
+bool encode_vec(CUtensorMap* m, const fit_grid* g, int nbatch, const void* base, int w, int h) {
+  const cuuint64_t ce = sizeof(T) / 4;  // 8-byte copy elements per complex value
+  const cuuint64_t dims[4] = {3 * ce * (cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, (cuuint64_t)nbatch};
+  const cuuint64_t rowb = 3 * ce * 8 * (cuuint64_t)g->nx;
+  const cuuint64_t str[3] = {rowb, rowb * g->ny, rowb * g->ny * g->nz};
+  const cuuint32_t box[4] = {(cuuint32_t)(3 * ce * w), (cuuint32_t)h, 1, 1};
+  return encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, base, dims, str, box);
+}
+
+// the arguments that do not depend on how the tiles are dealt out
+template <typename T>
+void fill_args(FusedArgs<T>& a, const fit_grid* g, int nbatch, const fit_omega& om, const void* x, int ty,
+               double out_scale) {
+  a.x = (const typename cplx<T>::t*)x;
+  a.ek = nullptr;
+  a.nxp = g->nxp;
+  a.omega = om.dev;
+  for (int b = 0; b < FIT_OMEGA_ARGS; ++b) a.om[b] = !om.dev && b < nbatch ? om.host[b] : 0.0;
+  a.err = g->err_dev;
+  a.abort = g->abort_dev;
+  a.abort_first = g->abort_mirror;
+  a.nx = g->nx;
+  a.ny = g->ny;
+  a.nz = g->nz;
+  a.ntx = (g->nx + TX - 1) / TX;
+  a.nty = (g->ny + ty - 1) / ty;
+  a.ne = g->ne;
+  a.out_scale = (T)out_scale;
+  a.nb = nbatch;
+  a.pf = 0;
+  a.flat = 0;
+}
+
+// Tiles of tz planes (tz <= 0: as many equal z-chunks per column as the resident CTAs allow) on one persistent wave.
+template <typename T>
+int tile_grid(FusedArgs<T>& a, fit_epi& e, int tz, long long slots) {
+  if (tz <= 0) {
+    const long long cols = (long long)a.ntx * a.nty * a.nb;
+    const long long per_col = std::max(1LL, slots / std::max(1LL, cols));
+    tz = (int)std::max(2LL, ((long long)a.nz + per_col - 1) / per_col);
+  }
+  a.flat = 0;
+  a.tz = tz;
+  a.nzc = (a.nz + tz - 1) / tz;
+  a.ntiles = a.ntx * a.nty * a.nzc * a.nb;
+  e.nslots = (long long)a.ntx * a.nty * a.nzc;
+  return (int)std::max(1LL, std::min((long long)a.ntiles, slots));
+}
+
+// launch of the CTA-synchronous kernel (complex64)
+template <int TY, int S>
+fit_status launch_sync(fit_grid* g, int nbatch, const fit_omega& om, const void* x, void* y, const float* nu,
+                       const float* ek, double out_scale, cudaStream_t s, fit_epi& e, int tz, int pf) {
+  CUtensorMap mx, my, mu, mnu, mek, mmask;
+  fit_status st = encode_coefs<float, TY>(g, nu, ek, &mnu, &mek, &mmask);
+  if (st != FIT_OK) return st;
+  const bool ku = e.mode == FIT_EPI_DOT_U || e.mode == FIT_EPI_RESID;
+  const void* ub = ku ? e.u : x;
+  // x with its halo; y (bulk tensor store) and the epilogue vector u by the tile's own cells
+  if (!encode_vec<float>(&mx, g, nbatch, x, TX + 4, TY + 2) || !encode_vec<float>(&my, g, nbatch, y, TX, TY) ||
+      ((uintptr_t)ub & 15) != 0 || !encode_vec<float>(&mu, g, nbatch, ub, TX, TY)) {
+    fit_set_error("fused apply: tensor map of a vector rejected");
+    return FIT_ECUDA;
+  }
+  FusedArgs<float> a;
+  fill_args(a, g, nbatch, om, x, TY, out_scale);
+  a.pf = pf;
+  const dim3 block(TX, TY, 1);
+  const int smem = ku ? Layout<TY, true>::smem(S) : Layout<TY, false>::smem(S);
+  auto run = [&](auto kern) -> fit_status {
+    FitResidency res;
+    FIT_CHECK_CUDA(fit_residency((const void*)kern, (int)(block.x * block.y), smem, &res));
+    const long long slots = res.ctas();
+    if (slots < 1) {  // shared memory or registers do not allow one resident CTA of this shape
+      fit_set_error("fused apply: launch shape does not fit on an SM");
+      return FIT_EINVAL;
+    }
+    const int grid = tile_grid(a, e, tz, slots);
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = programmatic_config(grid, block, smem, s, at);
+    FIT_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, mx, my, mu, mnu, mek, mmask, a, e));
+    return FIT_OK;
+  };
+  switch (e.mode) {
+    case FIT_EPI_NONE: return run(fused_apply_kernel<TY, FIT_EPI_NONE, S>);
+    case FIT_EPI_DOT_U: return run(fused_apply_kernel<TY, FIT_EPI_DOT_U, S>);
+    case FIT_EPI_DOT_TS: return run(fused_apply_kernel<TY, FIT_EPI_DOT_TS, S>);
+    case FIT_EPI_RESID: return run(fused_apply_kernel<TY, FIT_EPI_RESID, S>);
+    case FIT_EPI_DOT_XY: return run(fused_apply_kernel<TY, FIT_EPI_DOT_XY, S>);
+  }
+  fit_set_error("fused apply: unknown epilogue");
+  return FIT_EINVAL;
+}
+
 // launch of the warp-specialised kernel: R rows per consumer warp, NCW consumer warps, S stages
 template <typename T, int R, int NCW, int S, bool ODD>
 fit_status launch_rows(fit_grid* g, int nbatch, const fit_omega& om, const void* x, void* y, const T* nu,
@@ -1384,35 +1360,13 @@ fit_status launch_rows(fit_grid* g, int nbatch, const fit_omega& om, const void*
   if (st != FIT_OK) return st;
   if constexpr (ODD) {
     mx = mnu;  // (not used: rows of x come by plain bulk copies)
-  } else {
-    const cuuint64_t ce = L::CE;
-    const cuuint64_t dims[4] = {3 * ce * (cuuint64_t)g->nx, (cuuint64_t)g->ny, (cuuint64_t)g->nz, (cuuint64_t)nbatch};
-    const cuuint64_t rowb = 3 * ce * 8 * (cuuint64_t)g->nx;
-    const cuuint64_t str[3] = {rowb, rowb * g->ny, rowb * g->ny * g->nz};
-    const cuuint32_t box[4] = {(cuuint32_t)(3 * ce * (TX + 4)), TY + 2, 1, 1};
-    if (!encode(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, x, dims, str, box)) {
-      fit_set_error("fused apply: tensor map of x rejected");
-      return FIT_ECUDA;
-    }
+  } else if (!encode_vec<T>(&mx, g, nbatch, x, TX + 4, TY + 2)) {
+    fit_set_error("fused apply: tensor map of x rejected");
+    return FIT_ECUDA;
   }
   FusedArgs<T> a;
-  a.x = (const V*)x;
+  fill_args(a, g, nbatch, om, x, TY, out_scale);
   a.ek = ek;
-  a.nxp = g->nxp;
-  a.omega = om.dev;
-  for (int b = 0; b < FIT_OMEGA_ARGS; ++b) a.om[b] = !om.dev && b < nbatch ? om.host[b] : 0.0;
-  a.err = g->err_dev;
-  a.abort = g->abort_dev;
-  a.abort_first = g->abort_mirror;
-  a.nx = g->nx;
-  a.ny = g->ny;
-  a.nz = g->nz;
-  a.ntx = (g->nx + TX - 1) / TX;
-  a.nty = (g->ny + TY - 1) / TY;
-  a.ne = g->ne;
-  a.out_scale = (T)out_scale;
-  a.pf = 0;
-  a.nb = nbatch;
   constexpr int smem = L::smem();
   const dim3 block(TX, NCW + 2, 1);
   auto run = [&](auto kern) -> fit_status {
@@ -1424,25 +1378,14 @@ fit_status launch_rows(fit_grid* g, int nbatch, const fit_omega& om, const void*
       return FIT_EINVAL;
     }
     int grid = 0;
-    if (tz < 0 && nbatch == 1) {  // the (column, plane) pairs split evenly (see launch_variant)
+    if (tz < 0 && nbatch == 1) {  // the (column, plane) pairs cut into equal ranges, one per resident CTA
       const long long cap = (long long)a.ntx * a.nty * ((g->nz + 1) / 2);
       grid = (int)std::max(1LL, std::min(slots, cap));
       a.flat = 1;
       a.tz = a.nzc = a.ntiles = 0;
       e.nslots = grid;
     } else {
-      int tzz = tz;
-      if (tzz <= 0) {
-        const long long cols = (long long)a.ntx * a.nty * nbatch;
-        const long long per_col = std::max(1LL, slots / std::max(1LL, cols));
-        tzz = (int)std::max(2LL, ((long long)g->nz + per_col - 1) / per_col);
-      }
-      a.flat = 0;
-      a.tz = tzz;
-      a.nzc = (g->nz + tzz - 1) / tzz;
-      a.ntiles = a.ntx * a.nty * a.nzc * nbatch;
-      e.nslots = (long long)a.ntx * a.nty * a.nzc;
-      grid = (int)std::max(1LL, std::min((long long)a.ntiles, slots));
+      grid = tile_grid(a, e, tz, slots);
     }
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = programmatic_config(grid, block, smem, s, at);
@@ -1509,7 +1452,7 @@ fit_status launch_fused(fit_grid* g, int nbatch, const fit_omega& om, const void
     return with_sync_shape(
         v,
         [&](auto ty, auto st) {
-          return launch_variant<T, ty.value, st.value>(g, nbatch, om, x, y, nu, ek, out_scale, s, e, v.tz, v.pf);
+          return launch_sync<ty.value, st.value>(g, nbatch, om, x, y, nu, ek, out_scale, s, e, v.tz, v.pf);
         },
         FIT_EINVAL);
   }
@@ -1541,11 +1484,8 @@ int kernel_override(int* variant) {
   return 0;
 }
 
-bool fused_supported(const fit_grid* g, fit_prec prec) {
-  (void)g;
-  (void)prec;
-  return encoder() != nullptr;
-}
+// the fused kernels need the driver's tensor-map encoder
+bool fused_supported() { return encoder() != nullptr; }
 
 // tensor-map copies of x start on 16-byte boundaries only if a grid row holds a whole number of 16-byte
 // units; other grids (complex64, odd nx) run the warp-specialised kernel's plain row copies
@@ -1568,7 +1508,7 @@ int variant_smem(const Variant& v, bool ku) {
     return with_sync_shape(
         v,
         [&](auto ty, auto st) {
-          return ku ? Layout<T, ty.value, true>::smem(st.value) : Layout<T, ty.value, false>::smem(st.value);
+          return ku ? Layout<ty.value, true>::smem(st.value) : Layout<ty.value, false>::smem(st.value);
         },
         1 << 30);
   }
@@ -1667,7 +1607,7 @@ fit_status fit_tune_apply(fit_grid* g, int nbatch, const fit_omega& om, const vo
                           cudaStream_t s) {
   const long long key = (long long)nbatch * 2 + (prec == FIT_C64 ? 0 : 1);
   if (g->tuned.count(key)) return FIT_OK;
-  if (!fused_supported(g, prec)) {
+  if (!fused_supported()) {
     g->tuned[key] = -1;
     return FIT_OK;
   }
@@ -1791,7 +1731,7 @@ fit_status fit_launch_apply(fit_grid* g, int nbatch, const fit_omega& om, const 
   int forced = 0;
   const int ov = kernel_override(&forced);
   const bool aligned = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-  if (ov == 1 || !aligned || !fused_supported(g, prec))
+  if (ov == 1 || !aligned || !fused_supported())
     return launch_generic_kernel(g, nbatch, om, x, y, prec, out_scale, s, &e);
   if (ov == 2) return launch_choice(g, forced, nbatch, om, x, y, prec, out_scale, s, e);
   const long long key = (long long)nbatch * 2 + (prec == FIT_C64 ? 0 : 1);
@@ -1816,7 +1756,7 @@ fit_status fit_launch_apply_fixed(fit_grid* g, int nbatch, const fit_omega& om, 
                                   fit_prec prec, double out_scale, cudaStream_t s) {
   fit_epi e;
   const bool aligned = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-  if (!aligned || !fused_supported(g, prec))
+  if (!aligned || !fused_supported())
     return launch_generic_kernel(g, nbatch, om, x, y, prec, out_scale, s, &e);
   const long long key = (long long)nbatch * 2 + (prec == FIT_C64 ? 0 : 1);
   auto it = g->tuned.find(key);

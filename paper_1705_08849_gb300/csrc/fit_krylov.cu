@@ -2042,7 +2042,7 @@ struct Seq {
       zin = (const char*)w.Zb + (size_t)j * vecb;
     }
     apply(zin, wj1, FIT_EPI_NONE, nullptr, w.inner, st_inner);
-    // CGS2: each pass's last block reduces its partial sums (h, h2, then ||w||^2 and the Givens step)
+    // CGS2: each pass is followed by the sum of its blocks' partials (h, h2; then ||w||^2 with the Givens step)
     ortho<T, 0>(j, nullptr);
     ortho<T, 1>(j, w.h1);
     ortho<T, 2>(j, w.h2);
