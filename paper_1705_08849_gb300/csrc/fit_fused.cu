@@ -512,8 +512,8 @@ __device__ inline void named_barrier(int id, int nthreads) {
 //   complex64 (R = 1): HBM, behind the issue slots of 16 consumer warps per SM.  Sums and differences of
 //   complex values are single packed instructions (add.f32x2), an edge's coefficients come as 8-byte loads,
 //   and the epilogue vector is not staged: 300 -> about 250 instructions per 32 cells.  128^3, one system:
-//   38.2 -> 35.7 us per apply, 256 x 256 x 192: 199.7 -> 191.5 us (5.5 TB/s at 28 B per unknown), 96^3 x 8:
-//   93.3 -> 88.8 us.  Two rows per thread (4 + 2 / R fluxes instead of 6 + 1) leave half the warps and were
+//   38.9 -> 35.3 us per apply, 256 x 256 x 192: 200.1 -> 184.6 us (5.7 TB/s at 28 B per unknown), 96^3 x 8:
+//   95.4 -> 88.2 us.  Two rows per thread (4 + 2 / R fluxes instead of 6 + 1) leave half the warps and were
 //   slower: 39.2, 217 and 91 us.
 //   complex128 (R = 2): the FP64 pipe, two instructions per clock and SM.  The left column's fluxes come from
 //   the neighbouring lane by shuffle (the warp's first column gets its own from one flux evaluation that
@@ -1193,7 +1193,10 @@ struct Variant {
 // tz = -1 (warp-specialised kernel, one system): the (column, plane) pairs split evenly over the
 //         resident CTAs; with a batch it falls back to tz = 0
 // The CTA-synchronous kernel stays for grids of a few tiles, where a plane's way through the masking warp is
-// the longer one.
+// the longer one.  In complex128 the FP64 work of a step hides that way, and the shapes below are level with or
+// faster than its former CTA-synchronous ones from 10^3 cells up (16^3: 14.5 us in a graph, 16.4 before; 8 systems of
+// 25^3: 39.1 and 48.9); on fewer cells the generic kernel is the fastest by 1 to 2 us, which a search from a cold L2
+// does not always see.
 constexpr Variant kVariants64[] = {
     {8, 0, 4, 0, 1},  {8, -1, 4, 0, 1}, {8, 32, 4, 0, 1}, {8, 16, 4, 0, 1},
     // CTA-synchronous
@@ -1575,6 +1578,8 @@ static fit_status launch_choice(fit_grid* g, int choice, int nbatch, const fit_o
 // four-row tiles win throughout (a plane's rows are copied one by one, and three CTAs per SM overlap more of
 // them).  One system or few tiles: the even split, or balanced chunks; a batch with at least two waves of
 // 32-plane tiles: those, whose CTAs march in step over the systems of a column and share its coefficients in L2.
+// (Below about 45 000 cells in all the generic kernel is level, or up to 2 us faster when applies follow one another
+// in a graph; solves there run level on either.)
 // Best of all shapes against this rule: 15x17x13 10.8 / 10.8 us, 63x61x59 11.8 / 13.0, 149x107x83 33.7 / 33.7,
 // 255x251x191 235.7 / 241.8, 41x37x29 x 8 21.2 / 21.2, 95x97x93 x 8 134.3 / 134.3.  A search would cost the
 // first apply 34 ms.
