@@ -463,23 +463,23 @@ constexpr int VU = 2;
   _Pragma("unroll") for (int u = 0; u < VU; ++u) if (const long long e = e0 + u * es; e < (p).ne)
 
 // A thread's share of a dot product or norm.  How many terms that is depends on the grid of the pass, and so
-// on how many systems share the call: FP32 terms are added as a pair with the exact rounding error of every addition
-// (Knuth's two-sum), whose total carries one rounding whatever its length.  (Six FP32 additions a term, of which an
-// SM does 128 per clock while HBM brings it less than one element: COCG at 128^3 127.1 -> 127.8 us per iteration, 8
-// BiCGStab systems of 40x36x28 63.2 -> 64.0.)  FP64 terms are added plainly.
+// on how many systems share the call: FP32 terms are added with the rounding error of every addition carried into the
+// next (Kahan), which keeps the total within two roundings of the terms' absolute sum whatever its length.  (Four FP32
+// additions a term, of which an SM does 128 per clock while HBM brings it less than one element: COCG at 128^3
+// 127.4 -> 127.7 us per iteration, 8 BiCGStab systems of 40x36x28 62.9 -> 63.3.)  FP64 terms are added plainly.
 template <typename T>
 struct RunSum {
-  T hi = T(0), lo = T(0);
+  T sum = T(0), err = T(0);
   __device__ void add(T v) {
     if constexpr (sizeof(T) == 4) {
-      const T s = hi + v, w = s - hi;
-      lo += (hi - (s - w)) + (v - w);
-      hi = s;
+      const T y = v - err, s = sum + y;
+      err = (s - sum) - y;
+      sum = s;
     } else {
-      hi += v;
+      sum += v;
     }
   }
-  __device__ T value() const { return isfinite(hi) ? hi + lo : hi; }
+  __device__ T value() const { return sum; }
 };
 
 __global__ void __launch_bounds__(256) k_outer_init(const double2* __restrict__ rhs, double2* __restrict__ x,
